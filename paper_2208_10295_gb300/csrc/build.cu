@@ -11,6 +11,7 @@
 //      height; the first stops.  The root height bounds the traversal stack.
 #include "common.cuh"
 
+#include <type_traits>
 #include <utility>
 
 namespace lidar {
@@ -27,6 +28,13 @@ __device__ __forceinline__ int float_to_ordered(float f)
 __device__ __forceinline__ float ordered_to_float(int i)
 {
     return __int_as_float(i >= 0 ? i : i ^ 0x7FFFFFFF);
+}
+
+// Orders a bottom-up climb: the writes of a finished child before its arrival
+// at the parent, the arrival before the parent's reads (which go to L2).
+__device__ __forceinline__ void climb_fence()
+{
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
 }
 
 __device__ __forceinline__ float3 load_vert(const float* v, uint32_t i)
@@ -233,10 +241,11 @@ __global__ void __launch_bounds__(kBuildThreads) k_refit(const float4* __restric
     if (leaf >= n) return;
     int p = parent_leaf[leaf];
     while (p >= 0) {
-        __threadfence();
-        if (atomicAdd(&visits[p], 1) == 0) return;  // the sibling subtree is not finished yet
-        __threadfence();
-        float4 n3 = __ldcg(&nodes[4 * (int64_t)p + 3]);
+        const int before = atomicAdd(&visits[p], 1);
+        const float4 n3 = __ldcg(&nodes[4 * (int64_t)p + 3]);  // links and the next parent: nobody writes them here
+        const int next = parent_node[p];
+        if (before == 0) return;  // the sibling subtree is not finished yet
+        climb_fence();
         int cl = __float_as_int(n3.x), cr = __float_as_int(n3.y);
         Box L = cl < 0 ? leaf_box(tris, ~cl) : node_box(node_boxes, cl);
         Box R = cr < 0 ? leaf_box(tris, ~cr) : node_box(node_boxes, cr);
@@ -252,7 +261,8 @@ __global__ void __launch_bounds__(kBuildThreads) k_refit(const float4* __restric
         int h = 1 + max(hl, hr);
         heights[p] = h;
         if (p == 0) atomicMax(max_height, h);
-        p = parent_node[p];
+        climb_fence();
+        p = next;
     }
 }
 
@@ -974,7 +984,7 @@ cudaError_t collapse_bvh(cudaStream_t s, int width, const float4* binary_nodes, 
 // ---------------------------------------------------------------------------
 // Treelet restructuring of the binary hierarchy (Karras and Aila, "Fast
 // Parallel Construction of High-Quality Bounding Volume Hierarchies", HPG
-// 2013), written here for one thread per treelet.  Cost of a tree under the
+// 2013), one warp per treelet.  Cost of a tree under the
 // surface-area model: c_node x A(n) over its internal nodes plus c_tri x A(t)
 // over its triangles (A: half the surface area of the box).  One round climbs
 // the tree bottom-up (the second child to finish processes its parent, so a
@@ -1005,6 +1015,13 @@ struct TreeletArgs {
     const int* parent_leaf;   // [n_leaves]
     unsigned* visits;         // [n_binary] children finished, zero at the start of a round
     float* cost;              // [n_binary] surface-area cost of each node's subtree
+    // A treelet is a function of its subtree alone, so one that was kept and
+    // whose subtree is as it was is kept again without a look: mark[n] is the
+    // last round (1, 2, ...) that rewrote node n, up[n] the last one that
+    // rewrote a treelet of n's subtree before n was reached.
+    uint8_t* mark;            // [n_binary]
+    uint8_t* up;              // [n_binary]
+    int round;
     unsigned long long* changed;  // treelets rewritten in the round
     int* status;              // ST_BOUNDS: a child reference out of range, or a climb longer than the bound
     float c_node, c_tri;
@@ -1058,148 +1075,409 @@ __device__ __forceinline__ float subtree_cost(const TreeletArgs& a, int ref, con
     return ref < 0 ? a.c_tri * tbox_area(b, a.w) : __ldcg(&a.cost[ref]);
 }
 
-__device__ void treelet_node(const TreeletArgs& a, int node)
+// Subsets of a treelet's leaves by size (a bit mask each): the lanes of a warp
+// take the subsets of one size together, which depend on smaller sizes only.
+__device__ const unsigned char kSubsets2[21] = {3,  5,  6,  9,  10, 12, 17, 18, 20, 24, 33,
+                                                34, 36, 40, 48, 65, 66, 68, 72, 80, 96};
+__device__ const unsigned char kSubsets3[35] = {7,  11, 13, 14, 19, 21, 22, 25, 26, 28,  35, 37,
+                                                38, 41, 42, 44, 49, 50, 52, 56, 67, 69,  70, 73,
+                                                74, 76, 81, 82, 84, 88, 97, 98, 100, 104, 112};
+
+// One warp's treelet in shared memory.
+struct TreeletShared {
+    float box[6][kTreeletLeaves + 1];  // lo.x, hi.x, lo.y, hi.y, lo.z, hi.z of the leaves
+    float c[1 << kTreeletLeaves];      // c(S); before S is done, c_node x A(S)
+    unsigned char split[1 << kTreeletLeaves];
+    int ref[kTreeletLeaves + 1];       // the leaves
+    int inner[kTreeletLeaves + 1];     // the treelet's internal nodes, the root first
+    int out_s[kTreeletLeaves], out_id[kTreeletLeaves], out_ref[2][kTreeletLeaves];
+};
+
+// box of subset x of the treelet's leaves
+__device__ __forceinline__ TBox subset_box(const TreeletShared& t, int x)
 {
-    int lref[kTreeletLeaves];
-    TBox lbox[kTreeletLeaves];
-    float lcost[kTreeletLeaves];
-    int inner[kTreeletLeaves - 1];
-    treelet_child(a.nodes, node, 0, lref[0], lbox[0]);
-    treelet_child(a.nodes, node, 1, lref[1], lbox[1]);
-    if (!ref_ok(a, lref[0]) || !ref_ok(a, lref[1])) {
-        raise_status(a.status, ST_BOUNDS);
-        return;
-    }
-    lcost[0] = subtree_cost(a, lref[0], lbox[0]);
-    lcost[1] = subtree_cost(a, lref[1], lbox[1]);
-    TBox whole = lbox[0];
-    tbox_grow(whole, lbox[1]);
-    // the node's cost in its current shape
-    const float c_now = a.c_node * tbox_area(whole, a.w) + lcost[0] + lcost[1];
-    inner[0] = node;
-    int k = 2, n_inner = 1;
-    while (k < kTreeletLeaves) {
-        int best = -1;
-        float best_a = -1.0f;
-        for (int i = 0; i < k; ++i)
-            if (lref[i] >= 0 && tbox_area(lbox[i], a.w) > best_a) {
-                best_a = tbox_area(lbox[i], a.w);
-                best = i;
-            }
-        if (best < 0) break;
-        const int open = lref[best];
-        inner[n_inner++] = open;
-        treelet_child(a.nodes, open, 0, lref[best], lbox[best]);
-        treelet_child(a.nodes, open, 1, lref[k], lbox[k]);
-        if (!ref_ok(a, lref[best]) || !ref_ok(a, lref[k])) {
-            raise_status(a.status, ST_BOUNDS);
-            return;
+    TBox u;
+    bool first = true;
+    for (; x; x &= x - 1) {
+        const int i = __ffs(x) - 1;
+        TBox b;
+        for (int k = 0; k < 3; ++k) {
+            b.lo[k] = t.box[2 * k][i];
+            b.hi[k] = t.box[2 * k + 1][i];
         }
-        lcost[best] = subtree_cost(a, lref[best], lbox[best]);
-        lcost[k] = subtree_cost(a, lref[k], lbox[k]);
+        if (first) u = b;
+        else tbox_grow(u, b);
+        first = false;
+    }
+    return u;
+}
+
+// Cheapest partition of subset s (each once: the part with s's lowest leaf,
+// low | q for the proper submasks q of the others, largest q first, the first
+// of equal costs kept).  The lane tries q = v | fixed for the kTries submasks v
+// of `varied`; a subset whose partitions are spread over several lanes gives
+// each its own `fixed`.
+template <int kTries>
+__device__ __forceinline__ void best_partition(const TreeletShared& t, int s, int varied, int fixed, float& best,
+                                               int& bq)
+{
+    const int low = s & -s, rest = s ^ low;
+    best = INFINITY;
+    bq = 0;
+    int v = varied;
+#pragma unroll
+    for (int i = 0; i < kTries; ++i, v = (v - 1) & varied) {
+        const int q = v | fixed;
+        const float x = t.c[q | low] + t.c[s ^ (q | low)];
+        if (x < best && q != rest) {
+            best = x;
+            bq = q;
+        }
+    }
+}
+
+// lanes xor-partnered over `width` lanes agree on the cheapest (largest q of equal costs)
+__device__ __forceinline__ void merge_partition(float& best, int& bq, int width)
+{
+    for (int o = width / 2; o > 0; o >>= 1) {
+        const float b2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int q2 = __shfl_xor_sync(0xffffffffu, bq, o);
+        if (b2 < best || (b2 == best && q2 > bq)) {
+            best = b2;
+            bq = q2;
+        }
+    }
+}
+
+// The treelet at `node`, by one warp (all lanes call it).  Lane i < 7 holds the
+// treelet's leaf i while it grows; the areas of its 127 subsets are spread over
+// the lanes, four each; the dynamic program runs size by size, one subset per
+// lane up to five leaves, four lanes a subset at six, all lanes on the whole.
+// 1: rewritten, 0: kept, -1: a child reference out of range.
+//
+// A leaf that is an internal node has its own record in flight as soon as it
+// joins the treelet, so that opening it later waits for no load.
+__device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, int sub2, int sub3a, int sub3b)
+{
+    const int lane = threadIdx.x & 31;
+    constexpr unsigned kAll = 0xffffffffu;
+    float4 n0, n1, n2;       // this lane's leaf's record (the treelet's root at first)
+    int left, right;
+    auto fetch = [&](int r) {
+        n0 = __ldcg(&a.nodes[4 * (int64_t)r + 0]);
+        n1 = __ldcg(&a.nodes[4 * (int64_t)r + 1]);
+        n2 = __ldcg(&a.nodes[4 * (int64_t)r + 2]);
+        const int2 c = __ldcg(reinterpret_cast<const int2*>(&a.nodes[4 * (int64_t)r + 3]));
+        left = c.x;
+        right = c.y;
+    };
+    fetch(node);
+    int ref = lane == 0 ? left : (lane == 1 ? right : -1);
+    if (__any_sync(kAll, !ref_ok(a, ref))) return -1;
+    TBox box;
+    box.lo[0] = lane ? n1.x : n0.x; box.hi[0] = lane ? n1.y : n0.y;
+    box.lo[1] = lane ? n1.z : n0.z; box.hi[1] = lane ? n1.w : n0.w;
+    box.lo[2] = lane ? n2.z : n2.x; box.hi[2] = lane ? n2.w : n2.y;
+    float root_area;
+    {
+        TBox whole;
+        whole.lo[0] = fminf(n0.x, n1.x); whole.hi[0] = fmaxf(n0.y, n1.y);
+        whole.lo[1] = fminf(n0.z, n1.z); whole.hi[1] = fmaxf(n0.w, n1.w);
+        whole.lo[2] = fminf(n2.x, n2.z); whole.hi[2] = fmaxf(n2.y, n2.w);
+        root_area = tbox_area(whole, a.w);
+    }
+    float area = tbox_area(box, a.w);
+    float cost = a.c_tri * area;
+    if (lane < 2 && ref >= 0) {
+        fetch(ref);
+        cost = __ldcg(&a.cost[ref]);
+    }
+    const float first_cost = cost;  // lanes 0 and 1: the root's children
+    int k = 2, inner = node;        // lane j: the treelet's internal node j
+    while (k < kTreeletLeaves) {
+        // the internal leaf of largest area (ties to the lowest); areas are not
+        // negative, so their bits order like the values
+        const unsigned key = (lane < k && ref >= 0 && area > -1.0f) ? __float_as_uint(area) + 1u : 0u;
+        const unsigned top = __reduce_max_sync(kAll, key);
+        if (top == 0u) break;
+        const int best = __ffs(__ballot_sync(kAll, key == top)) - 1;
+        const int open = __shfl_sync(kAll, ref, best);
+        if (lane == k - 1) inner = open;
+        // side 0 stays in the opened leaf's lane, side 1 goes to lane k
+        const float bx = __shfl_sync(kAll, n1.x, best), by = __shfl_sync(kAll, n1.y, best);
+        const float bz = __shfl_sync(kAll, n1.z, best), bw = __shfl_sync(kAll, n1.w, best);
+        const float cz = __shfl_sync(kAll, n2.z, best), cw = __shfl_sync(kAll, n2.w, best);
+        const int rr = __shfl_sync(kAll, right, best);
+        const bool mine = lane == best || lane == k;
+        if (lane == best) {
+            box.lo[0] = n0.x; box.hi[0] = n0.y; box.lo[1] = n0.z; box.hi[1] = n0.w; box.lo[2] = n2.x; box.hi[2] = n2.y;
+            ref = left;
+        }
+        if (lane == k) {
+            box.lo[0] = bx; box.hi[0] = by; box.lo[1] = bz; box.hi[1] = bw; box.lo[2] = cz; box.hi[2] = cw;
+            ref = rr;
+        }
+        if (__any_sync(kAll, mine && !ref_ok(a, ref))) return -1;
+        if (mine) {
+            area = tbox_area(box, a.w);
+            if (ref >= 0) {
+                fetch(ref);
+                cost = __ldcg(&a.cost[ref]);
+            } else {
+                cost = a.c_tri * area;
+            }
+        }
         ++k;
     }
+    // the node's cost in its current shape
+    const float c_now = a.c_node * root_area + __shfl_sync(kAll, first_cost, 0) + __shfl_sync(kAll, first_cost, 1);
     if (k < 3) {
-        a.cost[node] = c_now;
-        return;
+        if (lane == 0) a.cost[node] = c_now;
+        return 0;
     }
-    // the cheapest binary tree over the k leaves: subsets in increasing order
-    // (every proper subset of S is smaller than S); each partition once (P
-    // holds S's lowest leaf)
-    float c[1 << kTreeletLeaves];
-    unsigned char split[1 << kTreeletLeaves];
+    __syncwarp();  // the treelet before this one is done with the shared arrays
+    if (lane < k) {
+        for (int j = 0; j < 3; ++j) {
+            t.box[2 * j][lane] = box.lo[j];
+            t.box[2 * j + 1][lane] = box.hi[j];
+        }
+        t.ref[lane] = ref;
+        if (lane < k - 1) t.inner[lane] = inner;
+    }
+    __syncwarp();
+    // areas: lane l takes the subsets 4 l + {0, 1, 2, 3}
     const int full = (1 << k) - 1;
-    for (int s = 1; s <= full; ++s) {
-        if ((s & (s - 1)) == 0) {
-            c[s] = lcost[__ffs(s) - 1];
-            split[s] = 0;
-            continue;
+    if (4 * lane <= full) {
+        TBox hi;
+        for (int j = 0; j < 3; ++j) {
+            hi.lo[j] = INFINITY;
+            hi.hi[j] = -INFINITY;
         }
-        TBox u;
-        bool first = true;
-        for (int i = 0; i < k; ++i)
-            if (s & (1 << i)) {
-                if (first) u = lbox[i];
-                else tbox_grow(u, lbox[i]);
-                first = false;
-            }
-        const int low = s & -s;
-        float best = INFINITY;
-        int bp = low;
-        for (int p = (s - 1) & s; p; p = (p - 1) & s) {
-            if (!(p & low)) continue;
-            const float v = c[p] + c[s ^ p];
-            if (v < best) {
-                best = v;
-                bp = p;
-            }
+#pragma unroll
+        for (int i = 2; i < kTreeletLeaves; ++i)
+            if ((lane >> (i - 2)) & 1)
+                for (int j = 0; j < 3; ++j) {
+                    hi.lo[j] = fminf(hi.lo[j], t.box[2 * j][i]);
+                    hi.hi[j] = fmaxf(hi.hi[j], t.box[2 * j + 1][i]);
+                }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            TBox u = hi;
+            for (int i = 0; i < 2; ++i)
+                if ((m >> i) & 1)
+                    for (int j = 0; j < 3; ++j) {
+                        u.lo[j] = fminf(u.lo[j], t.box[2 * j][i]);
+                        u.hi[j] = fmaxf(u.hi[j], t.box[2 * j + 1][i]);
+                    }
+            t.c[4 * lane + m] = a.c_node * tbox_area(u, a.w);
         }
-        c[s] = a.c_node * tbox_area(u, a.w) + best;
-        split[s] = (unsigned char)bp;
+    }
+    __syncwarp();
+    if (lane < k) t.c[1 << lane] = cost;
+    __syncwarp();
+    // up to five leaves: one subset per lane (those with leaves past k have none)
+    auto one = [&](int s, auto tries) {
+        if (s > full || s == 0) return;
+        float best;
+        int q;
+        best_partition<decltype(tries)::value>(t, s, s & (s - 1), 0, best, q);
+        t.c[s] += best;
+        t.split[s] = (unsigned char)(q | (s & -s));
+    };
+    one(sub2, std::integral_constant<int, 2>());
+    __syncwarp();
+    one(sub3a, std::integral_constant<int, 4>());
+    one(sub3b, std::integral_constant<int, 4>());
+    __syncwarp();
+    // subsets of four and five leaves are the complements of those of three and two
+    if (k >= 4) {
+        one(127 ^ sub3a, std::integral_constant<int, 8>());
+        one(sub3b ? 127 ^ sub3b : 0, std::integral_constant<int, 8>());
+        __syncwarp();
+    }
+    if (k >= 5) {
+        one(sub2 ? 127 ^ sub2 : 0, std::integral_constant<int, 16>());
+        __syncwarp();
+    }
+    if (k >= 6) {
+        // six leaves: four lanes a subset, each its own choice of the two highest leaves
+        const int s = lane < 28 ? 127 ^ (1 << (lane >> 2)) : 63;
+        const int rest = s & (s - 1);
+        const int b1 = 1 << (31 - __clz(rest)), b0 = 1 << (31 - __clz(rest ^ b1));
+        float best;
+        int q;
+        best_partition<8>(t, s, rest ^ b1 ^ b0, ((lane & 1) ? b0 : 0) | ((lane & 2) ? b1 : 0), best, q);
+        merge_partition(best, q, 4);
+        __syncwarp();
+        if (lane < 28 && (lane & 3) == 0 && s <= full) {
+            t.c[s] += best;
+            t.split[s] = (unsigned char)(q | (s & -s));
+        }
+        __syncwarp();
+    }
+    if (k == 7) {
+        float best;
+        int q;
+        best_partition<2>(t, 127, 2, lane << 2, best, q);
+        merge_partition(best, q, 32);
+        __syncwarp();
+        if (lane == 0) {
+            t.c[127] += best;
+            t.split[127] = (unsigned char)(q | 1);
+        }
+        __syncwarp();
     }
     // keep the current shape unless the optimum is clearly cheaper (it is
     // one of the shapes the program compares, so it is never dearer beyond
     // rounding)
-    if (!(c[full] < c_now * (1.0f - 1e-5f))) {
-        a.cost[node] = c_now;
-        return;
+    if (!(t.c[full] < c_now * (1.0f - 1e-5f))) {
+        if (lane == 0) a.cost[node] = c_now;
+        return 0;
     }
     // rewrite: subset S at internal node id, its parts as leaves or the next
-    // internal nodes of the treelet
-    int st_s[kTreeletLeaves], st_id[kTreeletLeaves];
-    int sp = 0, next = 1;
-    st_s[sp] = full;
-    st_id[sp++] = node;
-    while (sp > 0) {
-        --sp;
-        const int s = st_s[sp], id = st_id[sp];
-        const int part[2] = {split[s], s ^ split[s]};
-        int ref[2];
-        TBox box[2];
-        for (int side = 0; side < 2; ++side) {
-            const int x = part[side];
-            bool first = true;
-            for (int i = 0; i < k; ++i)
-                if (x & (1 << i)) {
-                    if (first) box[side] = lbox[i];
-                    else tbox_grow(box[side], lbox[i]);
-                    first = false;
+    // internal nodes of the treelet (one lane lays out the shape, then a lane
+    // a node writes it)
+    if (lane == 0) {
+        // the stack of subsets to place, eight bits each, in one register; a
+        // subset's internal node (of t.inner) goes along in the other
+        unsigned long long st = (unsigned long long)full, at = 0;
+        int next = 1;
+        for (int j = 0; j < k - 1; ++j) {
+            const int s = (int)(st & 0xFFu), id = (int)(at & 0xFFu);
+            st >>= 8;
+            at >>= 8;
+            const int p = t.split[s];
+            t.out_s[j] = s;
+            t.out_id[j] = t.inner[id];
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const int x = side ? s ^ p : p;
+                if ((x & (x - 1)) == 0) {
+                    t.out_ref[side][j] = t.ref[__ffs(x) - 1];
+                } else {
+                    t.out_ref[side][j] = t.inner[next];
+                    st = (st << 8) | (unsigned long long)x;
+                    at = (at << 8) | (unsigned long long)next;
+                    ++next;
                 }
-            if ((x & (x - 1)) == 0) {
-                ref[side] = lref[__ffs(x) - 1];
-            } else {
-                ref[side] = inner[next++];
-                st_s[sp] = x;
-                st_id[sp++] = ref[side];
             }
         }
-        const TBox& L = box[0];
-        const TBox& R = box[1];
+        atomicAdd(a.changed, 1ull);
+    }
+    __syncwarp();
+    if (lane < k - 1) {
+        const int s = t.out_s[lane], id = t.out_id[lane];
+        const TBox L = subset_box(t, t.split[s]), R = subset_box(t, s ^ t.split[s]);
         a.nodes[4 * (int64_t)id + 0] = make_float4(L.lo[0], L.hi[0], L.lo[1], L.hi[1]);
         a.nodes[4 * (int64_t)id + 1] = make_float4(R.lo[0], R.hi[0], R.lo[1], R.hi[1]);
         a.nodes[4 * (int64_t)id + 2] = make_float4(L.lo[2], L.hi[2], R.lo[2], R.hi[2]);
-        a.nodes[4 * (int64_t)id + 3] = make_float4(__int_as_float(ref[0]), __int_as_float(ref[1]), 0.0f, 0.0f);
-        a.cost[id] = c[s];
+        a.nodes[4 * (int64_t)id + 3] =
+            make_float4(__int_as_float(t.out_ref[0][lane]), __int_as_float(t.out_ref[1][lane]), 0.0f, 0.0f);
+        a.cost[id] = t.c[s];
+        a.mark[id] = (uint8_t)a.round;
     }
-    atomicAdd(a.changed, 1ull);
+    return 1;
 }
 
-__global__ void __launch_bounds__(128) k_treelet_round(TreeletArgs a)
+// One warp a block: warps end at very different times (most lanes stop after a
+// few steps, a few climb to the root), and a block's slot is only free when its
+// last warp ends.  16 a SM leaves 128 registers, without spills (0.65M
+// triangles, eight rounds, the whole build and a cast: 11.0 ms; four-warp
+// blocks 11.4 ms; 80 registers and 24 warps 11.3 ms, with spills).
+constexpr int kTreeletThreads = 32;
+constexpr int kTreeletBlocks = 16;
+
+// A lane per triangle climbs; the lanes that are second at their node have
+// the warp process those nodes' treelets one after another.
+//
+// What bounds it: the chain of each warp's treelets (issue ~40 %, ~1,000 warp
+// instructions and ~7,000 cycles a treelet) in the first round, and in later
+// ones, which look at few treelets, the climb itself (an arrival, a fence and
+// two loads a level).  Measured at 0.65M triangles (city, eight rounds): one
+// thread a treelet with its program in local memory 9.4 ms a round; by a warp
+// 1.2 ms; with the treelets whose subtree is unchanged kept unseen 1.2, 0.88,
+// 0.64, 0.51, 0.41, 0.35, 0.31, 0.30 ms.
+__global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_round(TreeletArgs a)
+{
+    __shared__ TreeletShared s_t[kTreeletThreads / 32];
+    TreeletShared& t = s_t[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int sub2 = lane < 21 ? kSubsets2[lane] : 0, sub3a = kSubsets3[lane], sub3b = lane < 3 ? kSubsets3[32 + lane] : 0;
+    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
+    int node = leaf < a.n_leaves ? a.parent_leaf[leaf] : -1;
+    for (int step = 0;; ++step) {
+        if (node >= a.n_binary || (node >= 0 && step >= kTreeletMaxClimb)) {
+            raise_status(a.status, ST_BOUNDS);
+            node = -1;
+        }
+        // what only this round's ancestors of the node may change is read
+        // beside the arrival, not after it
+        int2 c = make_int2(-1, -1);
+        int parent = -1;
+        bool look = false, below = false;  // the warp has to look at the treelet; its subtree changed this round
+        if (node >= 0) {
+            const unsigned before = atomicAdd(&a.visits[node], 1u);
+            c = __ldcg(reinterpret_cast<const int2*>(&a.nodes[4 * (int64_t)node + 3]));
+            parent = a.parent_node[node];
+            look = a.round == 1 || __ldcg(&a.mark[node]) == a.round - 1;
+            if (before == 0u) node = -1;  // the other child is still running
+        }
+        if (!__any_sync(0xffffffffu, node >= 0)) return;
+        climb_fence();  // the children's results are visible to the warp
+        __syncwarp();
+        if (node < 0) {
+            look = false;
+        } else if (!ref_ok(a, c.x) || !ref_ok(a, c.y)) {
+            raise_status(a.status, ST_BOUNDS);
+            look = false;
+        } else if (c.x < 0 && c.y < 0) {
+            // a pair of triangles has one shape: its lane notes the cost
+            if (look) {
+                int ref;
+                TBox L, R;
+                treelet_child(a.nodes, node, 0, ref, L);
+                treelet_child(a.nodes, node, 1, ref, R);
+                const float cost = subtree_cost(a, c.x, L), other = subtree_cost(a, c.y, R);
+                tbox_grow(L, R);
+                a.cost[node] = a.c_node * tbox_area(L, a.w) + cost + other;
+                look = false;
+            }
+        } else {
+            below = (c.x >= 0 && __ldcg(&a.up[c.x]) == a.round) || (c.y >= 0 && __ldcg(&a.up[c.y]) == a.round);
+            look = look || below;
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, look); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int did = treelet_node(a, __shfl_sync(0xffffffffu, node, src), t, sub2, sub3a, sub3b);
+            if (lane == src) {
+                if (did < 0) raise_status(a.status, ST_BOUNDS);
+                below = below || did > 0;
+            }
+        }
+        if (below) a.up[node] = (uint8_t)a.round;
+        climb_fence();  // every lane's writes, before a lane reports its node done
+        __syncwarp();
+        node = node >= 0 ? parent : -1;
+    }
+}
+
+// Height of the root: the longest climb of a leaf (a leaf's climb reads one
+// parent link a level, the upper ones from the caches, and needs no arrivals).
+__global__ void __launch_bounds__(kBuildThreads) k_root_height(const int* __restrict__ parent_node,
+                                                               const int* __restrict__ parent_leaf, int n_leaves,
+                                                               int n_binary, int* max_height, int* status)
 {
     const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (leaf >= a.n_leaves) return;
-    int node = a.parent_leaf[leaf];
-    for (int step = 0; node >= 0; ++step) {
-        if (node >= a.n_binary || step >= kTreeletMaxClimb) {
-            raise_status(a.status, ST_BOUNDS);
-            return;
+    int h = 0;
+    if (leaf < n_leaves)
+        for (int p = parent_leaf[leaf]; p >= 0; p = parent_node[p]) {
+            if (p >= n_binary || ++h > kTreeletMaxClimb) {
+                raise_status(status, ST_BOUNDS);
+                break;
+            }
         }
-        __threadfence();
-        if (atomicAdd(&a.visits[node], 1u) == 0u) return;  // the other child is still running
-        __threadfence();
-        treelet_node(a, node);
-        node = a.parent_node[node];
-    }
+    h = __reduce_max_sync(0xffffffffu, h);
+    if ((threadIdx.x & 31) == 0) atomicMax(max_height, h);
 }
 
 __global__ void k_parents_reset(int* parent_node, int n_binary)
@@ -1212,8 +1490,9 @@ __global__ void k_parents_reset(int* parent_node, int n_binary)
 
 size_t treelet_scratch_bytes(int64_t n_tris)
 {
-    // parents of nodes and leaves, visit counters, costs, heights, node boxes, counter
-    return 5 * align256(n_tris * sizeof(int)) + align256((size_t)n_tris * 2 * sizeof(float4)) + 256;
+    // parents of nodes and leaves, visit counters, costs, counter, marks
+    return 4 * align256(n_tris * sizeof(int)) + 256 +
+           2 * align256(n_tris);
 }
 
 cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, float4* nodes, int* max_height_dev,
@@ -1229,30 +1508,31 @@ cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, 
     int* parent_leaf = (int*)p; p += align256(n * sizeof(int));
     unsigned* visits = (unsigned*)p; p += align256(n * sizeof(int));
     float* cost = (float*)p; p += align256(n * sizeof(float));
-    int* heights = (int*)p; p += align256(n * sizeof(int));
-    float4* node_boxes = (float4*)p; p += align256((size_t)n * 2 * sizeof(float4));
-    unsigned long long* changed = (unsigned long long*)p;
+    unsigned long long* changed = (unsigned long long*)p; p += 256;
+    uint8_t* mark = (uint8_t*)p; p += align256(n);
+    uint8_t* up = (uint8_t*)p;
     const int nb_blocks = (n_binary + 255) / 256;
-    TreeletArgs a{tris, (int)n, n_binary, nodes, parent_node, parent_leaf, visits, cost, changed, status,
+    TreeletArgs a{tris, (int)n, n_binary, nodes, parent_node, parent_leaf, visits, cost, mark, up, 0, changed, status,
                   1.0f, tri_cost, area_w};
     cudaError_t e = cudaMemsetAsync(changed, 0, sizeof(unsigned long long), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(mark, 0, (size_t)((char*)up + n - (char*)mark), s);
     if (e != cudaSuccess) return e;
     for (int r = 0; r < rounds; ++r) {
+        a.round = r + 1;
         k_parents_reset<<<nb_blocks, 256, 0, s>>>(parent_node, n_binary);
         k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf);
         e = cudaMemsetAsync(visits, 0, (size_t)n_binary * sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
-        k_treelet_round<<<(int)((n + 127) / 128), 128, 0, s>>>(a);
+        k_treelet_round<<<(int)((n + kTreeletThreads - 1) / kTreeletThreads), kTreeletThreads, 0, s>>>(a);
     }
-    // parents, heights and the root height of the final shape (the boxes the
-    // refit writes are the same exact unions)
+    // parents and root height of the final shape (every box a rewrite stored is
+    // the exact union of the boxes below it)
     k_parents_reset<<<nb_blocks, 256, 0, s>>>(parent_node, n_binary);
     k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf);
-    e = cudaMemsetAsync(visits, 0, (size_t)n_binary * sizeof(unsigned), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(max_height_dev, 0, sizeof(int), s);
+    e = cudaMemsetAsync(max_height_dev, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    k_refit<<<(int)((n + kBuildThreads - 1) / kBuildThreads), kBuildThreads, 0, s>>>(
-        tris, n, nodes, node_boxes, heights, parent_node, parent_leaf, (int*)visits, max_height_dev);
+    k_root_height<<<(int)((n + kBuildThreads - 1) / kBuildThreads), kBuildThreads, 0, s>>>(
+        parent_node, parent_leaf, (int)n, n_binary, max_height_dev, status);
     e = cudaGetLastError();
     if (e == cudaSuccess && changed_host)
         e = cudaMemcpyAsync(changed_host, changed, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
