@@ -157,29 +157,39 @@ struct BuildScratch;
 cudaError_t build_lbvh(cudaStream_t s, const float* verts, int64_t n_verts, const uint32_t* tris,
                        const uint16_t* mat, const uint32_t* inst, int64_t n_tris, float4* nodes_out,
                        float4* tris_out, uint32_t* leaf_tri_out, int* status, int* max_depth_dev,
-                       void* scratch, size_t scratch_bytes, int method = 0, int ploc_radius = 16,
-                       AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
+                       void* scratch, size_t scratch_bytes, int num_sms, int coop, int method = 0,
+                       int ploc_radius = 16, AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
 // scratch of the clustering build (method 1), on top of nothing: it reuses build_lbvh's scratch
 size_t ploc_scratch_bytes(int64_t n_tris);
 size_t build_scratch_bytes(int64_t n_tris);
-// W-wide hierarchy (width 4 or 8) from the binary one (breadth-first,
-// deterministic); synchronises once per level.  `nodes` may be NULL to count
-// only.  *n_wide = wide nodes, *levels = height of the wide tree, *stack_need =
-// deepest traversal stack the tree can require.
+// The 4- and 8-wide hierarchies from the binary one (breadth-first,
+// deterministic): collapse_plan lists their nodes in scratch, collapse_write
+// writes one of them.  n_wide = wide nodes, levels = height of the wide tree,
+// stack_need = deepest traversal stack the tree can require.
 // sah_dp: children chosen by the SAH dynamic program (triangle test cost
 // tri_cost relative to a wide-node visit) instead of opening the largest child
-cudaError_t collapse_bvh(cudaStream_t s, int width, const float4* binary_nodes, int64_t n_binary, float4* nodes,
-                         int64_t* n_wide, int* levels, int* stack_need, void* scratch, size_t scratch_bytes,
-                         int sah_dp = 0, float tri_cost = 1.0f, AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
-size_t collapse_scratch_bytes(int64_t n_binary);
+struct WideInfo {
+    int n_wide, levels, stack_need, pad;
+};
+struct BuildResult {
+    int height;                   // of the binary tree
+    int pad;
+    unsigned long long treelets;  // rewritten by the restructuring
+    WideInfo wide[2];             // 4-wide, 8-wide
+};
+cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_binary, void* scratch,
+                          size_t scratch_bytes, int sah_dp, float tri_cost, AreaW area_w, int* status, int num_sms,
+                          int coop, WideInfo info_dev[2]);
+cudaError_t collapse_write(cudaStream_t s, int width, const float4* binary_nodes, int64_t n_binary, float4* nodes,
+                           int64_t n_wide, void* scratch, int sah_dp, AreaW area_w);
+size_t collapse_scratch_bytes(int64_t n_binary, int sah_dp);
 // treelet restructuring of the binary hierarchy (rounds > 0, n_tris >= 3);
-// recomputes the root height; *changed_host (valid after a stream
-// synchronisation) receives the number of treelets rewritten; a broken input
-// tree records ST_BOUNDS in *status
+// recomputes the root height; *treelets_dev receives the number of treelets
+// rewritten; a broken input tree records ST_BOUNDS in *status
 size_t treelet_scratch_bytes(int64_t n_tris);
 cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, float4* nodes, int* max_height_dev,
                                  int rounds, float tri_cost, void* scratch, size_t scratch_bytes,
-                                 unsigned long long* changed_host, int* status,
+                                 unsigned long long* treelets_dev, int* status,
                                  AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
 
 // sort.cu: stable LSD radix sort of (key, value) pairs, keys of `key_bits` bits

@@ -117,7 +117,7 @@ struct lidar_ctx {
     int num_sms = 0;
     int* status_dev = nullptr;
     unsigned long long* work_counter = nullptr;
-    int* aux_dev = nullptr;  // scratch ints (build height)
+    BuildResult* build_dev = nullptr;  // what a build leaves for the host (beside the status word)
     unsigned long long* adj_arrivals = nullptr;  // the one-pass adjoint's grid-wait counter (only grows)
     unsigned long long adj_arrivals_base = 0;    // its value once every launch so far has run
     int coop = 0;                 // the device launches cooperative kernels
@@ -251,7 +251,8 @@ lidar_status lidar_create(int device, void* cuda_stream, lidar_ctx** out)
     }
     c->status_dev = (int*)p;
     c->work_counter = (unsigned long long*)((char*)p + 64);
-    c->aux_dev = (int*)((char*)p + 128);
+    c->build_dev = (BuildResult*)((char*)p + 128);
+    static_assert(sizeof(BuildResult) <= 64, "fits between the work counter and the adjoint's");
     c->adj_arrivals = (unsigned long long*)((char*)p + 192);
     c->coop = coop;
     e = dev_alloc((void**)&c->sensors_dev, sizeof(SensorDev) * LIDAR_MAX_SENSORS);
@@ -361,7 +362,8 @@ lidar_status lidar_scene_build(lidar_ctx* c, const float* verts, int64_t n_verts
             return fail(LIDAR_ENOMEM);
         }
         s->bytes = s->n_nodes * 64 + s->n_nodes * 128 + n_tris * 48 + n_tris * 4;
-        lidar_status st = ensure_scratch(c, std::max({build_scratch_bytes(n_tris), collapse_scratch_bytes(s->n_nodes),
+        lidar_status st = ensure_scratch(c, std::max({build_scratch_bytes(n_tris),
+                                                      collapse_scratch_bytes(s->n_nodes, c->collapse),
                                                       c->build_method == 1 ? ploc_scratch_bytes(n_tris) : (size_t)0,
                                                       c->treelet_rounds > 0 ? treelet_scratch_bytes(n_tris) : (size_t)0}));
         if (st != LIDAR_OK) return fail(st);
@@ -373,56 +375,68 @@ lidar_status lidar_scene_build(lidar_ctx* c, const float* verts, int64_t n_verts
         cudaEvent_t e0 = ev.a, e1 = ev.b;
         cudaEventRecord(e0, c->stream);
         cudaError_t e = build_lbvh(c->stream, verts, n_verts, tris, mat, inst, n_tris, s->nodes, s->tris,
-                                   s->leaf_tri, c->status_dev, c->aux_dev, c->scratch, c->scratch_bytes,
-                                   n_tris >= 2 ? c->build_method : 0, c->ploc_radius, c->area_w);
-        unsigned long long treelets = 0;
+                                   s->leaf_tri, c->status_dev, &c->build_dev->height, c->scratch, c->scratch_bytes,
+                                   c->num_sms, c->coop, n_tris >= 2 ? c->build_method : 0, c->ploc_radius, c->area_w);
         if (e == cudaSuccess && c->treelet_rounds > 0)
-            e = restructure_treelets(c->stream, s->tris, n_tris, s->nodes, c->aux_dev, c->treelet_rounds, c->tri_cost,
-                                     c->scratch, c->scratch_bytes, &treelets, c->status_dev, c->area_w);
+            e = restructure_treelets(c->stream, s->tris, n_tris, s->nodes, &c->build_dev->height, c->treelet_rounds,
+                                     c->tri_cost, c->scratch, c->scratch_bytes, &c->build_dev->treelets, c->status_dev,
+                                     c->area_w);
+        if (e == cudaSuccess)
+            e = collapse_plan(c->stream, s->nodes, s->n_nodes, c->scratch, c->scratch_bytes, c->collapse, c->tri_cost,
+                              c->area_w, c->status_dev, c->num_sms, c->coop, c->build_dev->wide);
         cudaEventRecord(e1, c->stream);
         if (e != cudaSuccess) {
             set_error(std::string("lidar_scene_build: ") + cudaGetErrorString(e));
             return fail(LIDAR_ECUDA);
         }
-        if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
+        // one copy brings the status word and what the build left beside it
+        char head[256];
+        if (cudaMemcpyAsync(head, c->status_dev, sizeof(head), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+            cudaStreamSynchronize(c->stream) != cudaSuccess) {
             set_error("lidar_scene_build: stream synchronisation failed");
             return fail(LIDAR_ECUDA);
         }
         float ms = 0.0f;
         cudaEventElapsedTime(&ms, e0, e1);
         s->build_ms = ms;
-        s->treelets = (int64_t)treelets;
-        int w = 0, h = 0;
-        cudaMemcpy(&w, c->status_dev, sizeof(int), cudaMemcpyDeviceToHost);
-        cudaMemcpy(&h, c->aux_dev, sizeof(int), cudaMemcpyDeviceToHost);
-        cudaMemset(c->status_dev, 0, sizeof(int));
-        s->max_depth = h;
+        int w = 0;
+        BuildResult built;
+        memcpy(&w, head, sizeof(int));
+        memcpy(&built, head + ((char*)c->build_dev - (char*)c->status_dev), sizeof(built));
+        if (w != ST_OK) cudaMemsetAsync(c->status_dev, 0, sizeof(int), c->stream);
+        s->treelets = c->treelet_rounds > 0 ? (int64_t)built.treelets : 0;
+        s->max_depth = built.height;
         if (w != ST_OK) return fail(status_from_word(w));
-        if (h > kTraversalStack) {
-            set_error("lidar_scene_build: BVH height " + std::to_string(h) + " exceeds the traversal stack (" +
-                      std::to_string(kTraversalStack) + ")");
+        if (built.height > kTraversalStack) {
+            set_error("lidar_scene_build: BVH height " + std::to_string(built.height) +
+                      " exceeds the traversal stack (" + std::to_string(kTraversalStack) + ")");
             return fail(LIDAR_ESTACK);
         }
+        const WideInfo& w4 = built.wide[0];
+        const WideInfo& w8 = built.wide[1];
+        if (w4.stack_need > kTraversalStack) {
+            set_error("lidar_scene_build: 4-wide BVH could need " + std::to_string(w4.stack_need) +
+                      " stack entries, more than the traversal stack (" + std::to_string(kTraversalStack) + ")");
+            return fail(LIDAR_ESTACK);
+        }
+        // the 8-wide tree gets an exact allocation; one that could need more
+        // than the traversal stack is not kept (the 4-wide and binary ones serve)
+        const bool keep8 = w8.stack_need <= kTraversalStack && w8.n_wide > 0;
+        if (keep8 && dev_alloc((void**)&s->nodes8, (size_t)w8.n_wide * 16 * sizeof(float4)) != cudaSuccess) {
+            cudaGetLastError();
+            set_error("lidar_scene_build: device allocation failed (8-wide tree)");
+            return fail(LIDAR_ENOMEM);
+        }
         cudaEventRecord(e0, c->stream);
-        int need4 = 0;
-        cudaError_t e4 = collapse_bvh(c->stream, 4, s->nodes, s->n_nodes, s->nodes4, &s->n_nodes4, &s->levels4,
-                                      &need4, c->scratch, c->scratch_bytes, c->collapse, c->tri_cost, c->area_w);
-        // the 8-wide tree: count its nodes and the stack it could need, then
-        // write it into an exact allocation; a tree that could need more than
-        // the traversal stack is not kept (the 4-wide and binary ones serve)
-        int64_t n8 = 0;
-        int levels8 = 0, need8 = 0;
-        if (e4 == cudaSuccess)
-            e4 = collapse_bvh(c->stream, 8, s->nodes, s->n_nodes, nullptr, &n8, &levels8, &need8, c->scratch,
-                              c->scratch_bytes, c->collapse, c->tri_cost, c->area_w);
-        if (e4 == cudaSuccess && need8 <= kTraversalStack && n8 > 0) {
-            if (dev_alloc((void**)&s->nodes8, (size_t)n8 * 16 * sizeof(float4)) != cudaSuccess) {
-                cudaGetLastError();
-                set_error("lidar_scene_build: device allocation failed (8-wide tree)");
-                return fail(LIDAR_ENOMEM);
-            }
-            e4 = collapse_bvh(c->stream, 8, s->nodes, s->n_nodes, s->nodes8, &s->n_nodes8, &s->levels8, &need8,
-                              c->scratch, c->scratch_bytes, c->collapse, c->tri_cost, c->area_w);
+        cudaError_t e4 = collapse_write(c->stream, 4, s->nodes, s->n_nodes, s->nodes4, w4.n_wide, c->scratch,
+                                        c->collapse, c->area_w);
+        s->n_nodes4 = w4.n_wide;
+        s->levels4 = w4.levels;
+        if (e4 == cudaSuccess && keep8) {
+            e4 = collapse_write(c->stream, 8, s->nodes, s->n_nodes, s->nodes8, w8.n_wide, c->scratch, c->collapse,
+                                c->area_w);
+            s->n_nodes8 = w8.n_wide;
+            s->levels8 = w8.levels;
             s->bytes += s->n_nodes8 * 256;
         }
         cudaEventRecord(e1, c->stream);
@@ -432,11 +446,6 @@ lidar_status lidar_scene_build(lidar_ctx* c, const float* verts, int64_t n_verts
         }
         cudaEventElapsedTime(&ms, e0, e1);
         s->build_ms += ms;
-        if (need4 > kTraversalStack) {
-            set_error("lidar_scene_build: 4-wide BVH could need " + std::to_string(need4) +
-                      " stack entries, more than the traversal stack (" + std::to_string(kTraversalStack) + ")");
-            return fail(LIDAR_ESTACK);
-        }
     }
     c->scenes.insert(s);
     *out = s;
