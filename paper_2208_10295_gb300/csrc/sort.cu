@@ -1,13 +1,20 @@
 // Stable LSD radix sort of (key, value) pairs, hand-written.
 //
-// Each pass sorts by one 4-bit digit with three kernels ("reduce, then scan,
+// Each pass sorts by one 8-bit digit with three kernels ("reduce, then scan,
 // then scatter"):
-//   upsweep   : per tile digit histogram, written digit-major [16][n_tiles]
-//   scan      : one block turns the histogram into exclusive global offsets
-//   downsweep : per tile stable ranking (warp match + cross-warp prefix per
-//               round of 256 keys) and scatter to offset[digit][tile] + rank.
-// Keys are read in a striped layout (key index = tile*TILE + round*256 + tid),
-// so ordering by (round, warp, lane) is the input order and the pass is stable.
+//   upsweep   : per tile digit histogram, written digit-major [256][n_tiles]
+//   scan      : one block per digit turns its row into exclusive offsets and
+//               leaves the digit's total
+//   downsweep : per tile stable ranking and scatter to the digit's base + the
+//               tile's offset + rank
+// A warp takes kSortItems x 32 consecutive keys of the tile, 32 at a time, so
+// ordering by (warp, step, lane) is the input order and the pass is stable.
+// Up to kSmallSort pairs one block sorts in shared memory, in one launch.
+//
+// What bounds it: launches and latency (1M pairs are 12 MB, in L2 all along).
+// 4-bit digits took 16 passes, with a block-wide barrier per 256 keys and all
+// counts scanned by one block: 0.51 ms for 1M 63-bit keys; 8-bit digits, eight
+// passes ranked warp by warp and a scan block per digit: 0.23 ms.
 #include "common.cuh"
 
 namespace lidar {
@@ -16,66 +23,94 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
-constexpr int kRadixBits = 4;
+constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kSortWarps = kSortThreads / 32;
+
+template <typename K>
+__device__ __forceinline__ uint32_t digit_of(K key, int shift)
+{
+    return (uint32_t)(key >> shift) & (uint32_t)(kRadix - 1);
+}
+
+// lanes of the warp with the same digit (the ones past the end form a group of their own)
+__device__ __forceinline__ uint32_t peers_of(uint32_t dg)
+{
+    return __match_any_sync(0xffffffffu, dg);
+}
 
 template <typename K>
 __global__ void __launch_bounds__(kSortThreads) k_upsweep(const K* __restrict__ keys, int64_t n, int shift,
                                                           int n_tiles, uint32_t* __restrict__ counts)
 {
     __shared__ uint32_t s_cnt[kRadix];
-    if (threadIdx.x < kRadix) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
+    s_cnt[threadIdx.x] = 0;
+    const int lane = threadIdx.x & 31;
     const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    uint32_t local[kRadix];
-#pragma unroll
-    for (int d = 0; d < kRadix; ++d) local[d] = 0;
+    uint32_t dg[kSortItems];
 #pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
-        int64_t idx = base + (int64_t)i * kSortThreads + threadIdx.x;
-        if (idx < n) {
-            uint32_t dg = (uint32_t)(keys[idx] >> shift) & (kRadix - 1);
-#pragma unroll
-            for (int d = 0; d < kRadix; ++d) local[d] += (dg == (uint32_t)d);
-        }
-    }
-    // warp-reduce each digit count, one shared atomic per warp and digit
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int d = 0; d < kRadix; ++d) {
-        uint32_t v = local[d];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0 && v) atomicAdd(&s_cnt[d], v);
+        const int64_t idx = base + (int64_t)i * kSortThreads + threadIdx.x;
+        dg[i] = idx < n ? digit_of(keys[idx], shift) : (uint32_t)kRadix;
     }
     __syncthreads();
-    if (threadIdx.x < kRadix) counts[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = s_cnt[threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const uint32_t peers = peers_of(dg[i]);
+        if (dg[i] < (uint32_t)kRadix && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[dg[i]], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+    counts[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = s_cnt[threadIdx.x];
 }
 
-// Exclusive scan of `n` counts in place, one block of 1024 threads.
-__global__ void __launch_bounds__(1024) k_scan_counts(uint32_t* __restrict__ counts, int64_t n)
+// Exclusive scan of one digit's counts in place; its total to totals[digit].
+__global__ void __launch_bounds__(kSortThreads) k_scan_digit(uint32_t* __restrict__ counts, int n_tiles,
+                                                             uint32_t* __restrict__ totals)
 {
-    __shared__ uint32_t s_sum[1024];
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t lo = (int64_t)threadIdx.x * per;
-    const int64_t hi = min(lo + per, n);
-    uint32_t s = 0;
-    for (int64_t i = lo; i < hi; ++i) s += counts[i];
-    s_sum[threadIdx.x] = s;
+    __shared__ uint32_t s_sum[kSortWarps];
+    uint32_t* row = counts + (int64_t)blockIdx.x * n_tiles;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    for (int base = 0; base < n_tiles; base += kSortThreads) {
+        const int i = base + threadIdx.x;
+        const uint32_t v = i < n_tiles ? row[i] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        __syncthreads();
+        if (lane == 31) s_sum[warp] = x;
+        __syncthreads();
+        uint32_t before = 0, sum = 0;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const uint32_t y = s_sum[w];
+            if (w < warp) before += y;
+            sum += y;
+        }
+        if (i < n_tiles) row[i] = carry + before + x - v;
+        carry += sum;
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
+}
+
+// exclusive prefix over the 256 threads of a block
+__device__ __forceinline__ uint32_t digit_prefix(uint32_t v, uint32_t* s_sum)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_sum[warp] = x;
     __syncthreads();
-    // Hillis-Steele inclusive scan over the 1024 partial sums
-    for (int off = 1; off < 1024; off <<= 1) {
-        uint32_t v = (threadIdx.x >= (unsigned)off) ? s_sum[threadIdx.x - off] : 0u;
-        __syncthreads();
-        s_sum[threadIdx.x] += v;
-        __syncthreads();
-    }
-    uint32_t run = (threadIdx.x == 0) ? 0u : s_sum[threadIdx.x - 1];
-    for (int64_t i = lo; i < hi; ++i) {
-        uint32_t c = counts[i];
-        counts[i] = run;
-        run += c;
-    }
+    uint32_t before = 0;
+    for (int w = 0; w < warp; ++w) before += s_sum[w];
+    return before + x - v;
 }
 
 template <typename K>
@@ -84,49 +119,183 @@ __global__ void __launch_bounds__(kSortThreads) k_downsweep(const K* __restrict_
                                                             K* __restrict__ keys_out,
                                                             uint32_t* __restrict__ vals_out, int64_t n,
                                                             int shift, int n_tiles,
-                                                            const uint32_t* __restrict__ offsets)
+                                                            const uint32_t* __restrict__ offsets,
+                                                            const uint32_t* __restrict__ totals)
 {
-    __shared__ uint32_t s_off[kRadix];
-    __shared__ uint32_t s_base[kRadix];
-    __shared__ uint32_t s_wcnt[kSortWarps][kRadix];
+    __shared__ uint32_t s_at[kSortWarps][kRadix];  // per warp: keys of a digit so far, then where its next ones go
+    __shared__ uint32_t s_out[kRadix];
+    __shared__ K s_key[kSortTile];
+    __shared__ uint32_t s_val[kSortTile];
+    __shared__ uint32_t s_sum[kSortWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x < kRadix) {
-        s_off[threadIdx.x] = offsets[(int64_t)threadIdx.x * n_tiles + blockIdx.x];
-        s_base[threadIdx.x] = 0;
+    const uint32_t total = totals[threadIdx.x];
+    const uint32_t tile_off = offsets[(int64_t)threadIdx.x * n_tiles + blockIdx.x];
+    const int64_t base = (int64_t)blockIdx.x * kSortTile + warp * (32 * kSortItems) + lane;
+    K key[kSortItems];
+    uint32_t val[kSortItems], rank[kSortItems];
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int64_t idx = base + i * 32;
+        key[i] = idx < n ? keys_in[idx] : (K)0;
+        val[i] = idx < n ? vals_in[idx] : 0u;
     }
-    if (threadIdx.x < kSortWarps * kRadix) (&s_wcnt[0][0])[threadIdx.x] = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) s_at[w][threadIdx.x] = 0;
     __syncthreads();
     const uint32_t lt_mask = (1u << lane) - 1u;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+#pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
-        int64_t idx = base + (int64_t)i * kSortThreads + threadIdx.x;
-        const bool ok = idx < n;
-        K key = ok ? keys_in[idx] : (K)0;
-        uint32_t val = ok ? vals_in[idx] : 0u;
-        uint32_t dg = ok ? ((uint32_t)(key >> shift) & (kRadix - 1)) : (uint32_t)kRadix;
-        uint32_t peers = __match_any_sync(0xffffffffu, dg);
-        uint32_t wrank = __popc(peers & lt_mask);
-        if (ok && wrank == 0) s_wcnt[warp][dg] = __popc(peers);
+        const bool ok = base + i * 32 < n;
+        const uint32_t dg = ok ? digit_of(key[i], shift) : (uint32_t)kRadix;
+        const uint32_t peers = peers_of(dg);
+        rank[i] = 0;
+        if (ok) rank[i] = s_at[warp][dg] + __popc(peers & lt_mask);
+        __syncwarp();
+        if (ok && lane == __ffs(peers) - 1) s_at[warp][dg] += __popc(peers);
+        __syncwarp();
+    }
+    // thread d: digit d's first place in the sorted tile and of each warp's
+    // share, and how far from there the output is
+    const uint32_t first = digit_prefix(total, s_sum) + tile_off;  // (its barrier ends the counting)
+    uint32_t mine = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+        const uint32_t c = s_at[w][threadIdx.x];
+        s_at[w][threadIdx.x] = mine;
+        mine += c;
+    }
+    __syncthreads();
+    const uint32_t local = digit_prefix(mine, s_sum);
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) s_at[w][threadIdx.x] += local;
+    s_out[threadIdx.x] = first - local;
+    __syncthreads();
+    // sorted in shared memory first, so that a digit's keys leave side by side
+    // (scattered from registers: 19 us a pass for 1M pairs, against 15)
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        if (base + i * 32 >= n) continue;
+        const uint32_t pos = s_at[warp][digit_of(key[i], shift)] + rank[i];
+        s_key[pos] = key[i];
+        s_val[pos] = val[i];
+    }
+    __syncthreads();
+    const int count = (int)min((int64_t)kSortTile, n - (int64_t)blockIdx.x * kSortTile);
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int k = i * kSortThreads + threadIdx.x;
+        if (k >= count) break;
+        const K x = s_key[k];
+        const uint32_t pos = s_out[digit_of(x, shift)] + k;
+        keys_out[pos] = x;
+        vals_out[pos] = s_val[k];
+    }
+}
+
+// Up to kSmallSort pairs in one block: every pass ranks out of registers and
+// scatters through shared memory.  (770 pairs of 63-bit keys: 24 launches
+// would take 55 us; 48 launches of 4-bit passes took 270 us, this one 16.)
+constexpr int kSmallSort = 4096;
+constexpr int kSmallThreads = 512;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallItems = kSmallSort / kSmallThreads;
+
+template <typename K>
+constexpr size_t small_sort_smem()
+{
+    return kSmallSort * (sizeof(K) + sizeof(uint32_t)) + kSmallWarps * kRadix * sizeof(uint32_t);
+}
+
+template <typename K>
+__global__ void __launch_bounds__(kSmallThreads) k_sort_small(K* __restrict__ keys, uint32_t* __restrict__ vals, int n,
+                                                              int key_bits)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    K* s_key = (K*)smem;
+    uint32_t* s_val = (uint32_t*)(s_key + kSmallSort);
+    uint32_t(*s_at)[kRadix] = (uint32_t(*)[kRadix])(s_val + kSmallSort);
+    __shared__ uint32_t s_sum[kRadix / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the fewest whole steps of 32 per warp that hold n
+    const int items = (n + kSmallThreads - 1) / kSmallThreads;
+    const int base = warp * (32 * items) + lane;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    K key[kSmallItems];
+    uint32_t val[kSmallItems], rank[kSmallItems];
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int idx = base + i * 32;
+        const bool ok = i < items && idx < n;
+        key[i] = ok ? keys[idx] : (K)0;
+        val[i] = ok ? vals[idx] : 0u;
+    }
+    for (int shift = 0; shift < key_bits; shift += kRadixBits) {
+        for (int k = threadIdx.x; k < kSmallWarps * kRadix; k += kSmallThreads) (&s_at[0][0])[k] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            if (i >= items) break;
+            const bool ok = base + i * 32 < n;
+            const uint32_t dg = ok ? digit_of(key[i], shift) : (uint32_t)kRadix;
+            const uint32_t peers = peers_of(dg);
+            rank[i] = 0;
+            if (ok) rank[i] = s_at[warp][dg] + __popc(peers & lt_mask);
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) s_at[warp][dg] += __popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        // thread d < 256: counts before each warp, then the digit's base added
+        uint32_t total = 0, x = 0;
+        if (threadIdx.x < kRadix) {
+#pragma unroll
+            for (int w = 0; w < kSmallWarps; ++w) {
+                const uint32_t c = s_at[w][threadIdx.x];
+                s_at[w][threadIdx.x] = total;
+                total += c;
+            }
+            x = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) s_sum[warp] = x;
+        }
         __syncthreads();
         if (threadIdx.x < kRadix) {
-            uint32_t run = s_base[threadIdx.x];
+            uint32_t first = x - total;
+            for (int w = 0; w < warp; ++w) first += s_sum[w];
 #pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) {
-                uint32_t c = s_wcnt[w][threadIdx.x];
-                s_wcnt[w][threadIdx.x] = run;
-                run += c;
+            for (int w = 0; w < kSmallWarps; ++w) s_at[w][threadIdx.x] += first;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            if (i >= items) break;
+            if (base + i * 32 < n) {
+                const uint32_t pos = s_at[warp][digit_of(key[i], shift)] + rank[i];
+                s_key[pos] = key[i];
+                s_val[pos] = val[i];
             }
-            s_base[threadIdx.x] = run;
         }
         __syncthreads();
-        if (ok) {
-            uint32_t pos = s_off[dg] + s_wcnt[warp][dg] + wrank;
-            keys_out[pos] = key;
-            vals_out[pos] = val;
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            const int idx = base + i * 32;
+            if (i < items && idx < n) {
+                key[i] = s_key[idx];
+                val[i] = s_val[idx];
+            }
         }
-        __syncthreads();
-        if (threadIdx.x < kSortWarps * kRadix) (&s_wcnt[0][0])[threadIdx.x] = 0;
-        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int idx = base + i * 32;
+        if (i < items && idx < n) {
+            keys[idx] = key[i];
+            vals[idx] = val[i];
+        }
     }
 }
 
@@ -136,12 +305,21 @@ cudaError_t radix_sort_pairs(cudaStream_t s, K* keys, uint32_t* vals, int64_t n,
 {
     if (n <= 1) return cudaSuccess;
     if (scratch_bytes < radix_sort_scratch_bytes(n)) return cudaErrorInvalidValue;
+    if (n <= kSmallSort) {
+        constexpr size_t smem = small_sort_smem<K>();
+        cudaError_t e = cudaFuncSetAttribute(k_sort_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_sort_small<K><<<1, kSmallThreads, smem, s>>>(keys, vals, (int)n, key_bits);
+        return cudaGetLastError();
+    }
     const int n_tiles = (int)((n + kSortTile - 1) / kSortTile);
     char* p = (char*)scratch;
     K* alt_keys = (K*)p;
     p += ((n * sizeof(uint64_t) + 255) / 256) * 256;
     uint32_t* alt_vals = (uint32_t*)p;
     p += ((n * sizeof(uint32_t) + 255) / 256) * 256;
+    uint32_t* totals = (uint32_t*)p;
+    p += kRadix * sizeof(uint32_t);
     uint32_t* counts = (uint32_t*)p;
     const int passes = (key_bits + kRadixBits - 1) / kRadixBits;
     K* kin = keys;
@@ -151,8 +329,8 @@ cudaError_t radix_sort_pairs(cudaStream_t s, K* keys, uint32_t* vals, int64_t n,
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = pass * kRadixBits;
         k_upsweep<K><<<n_tiles, kSortThreads, 0, s>>>(kin, n, shift, n_tiles, counts);
-        k_scan_counts<<<1, 1024, 0, s>>>(counts, (int64_t)kRadix * n_tiles);
-        k_downsweep<K><<<n_tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, n_tiles, counts);
+        k_scan_digit<<<kRadix, kSortThreads, 0, s>>>(counts, n_tiles, totals);
+        k_downsweep<K><<<n_tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, n_tiles, counts, totals);
         K* tk = kin; kin = kout; kout = tk;
         uint32_t* tv = vin; vin = vout; vout = tv;
     }
@@ -169,7 +347,7 @@ size_t radix_sort_scratch_bytes(int64_t n)
 {
     const int64_t n_tiles = (n + kSortTile - 1) / kSortTile;
     return ((n * sizeof(uint64_t) + 255) / 256) * 256 + ((n * sizeof(uint32_t) + 255) / 256) * 256 +
-           (size_t)kRadix * n_tiles * sizeof(uint32_t) + 256;
+           (size_t)kRadix * (n_tiles + 1) * sizeof(uint32_t) + 256;
 }
 
 cudaError_t radix_sort_pairs_u64(cudaStream_t s, uint64_t* keys, uint32_t* vals, int64_t n, int key_bits,
