@@ -362,37 +362,68 @@ __device__ __forceinline__ float union_half_area(float4 alo, float4 ahi, float4 
 
 constexpr uint64_t kBuildWaitNs = 2000000000ull;
 
-// The `blocks` blocks of a cooperative launch meet for the phase-th time
-// (`counter` is zero before the launch); one block alone only meets its own
-// threads.  Bounded: after two seconds ST_TIMEOUT, and false in every thread.
-__device__ bool build_barrier(unsigned* counter, unsigned blocks, unsigned& phase, int* status)
+
+// Where the blocks of a cooperative launch meet: a counter they arrive at and
+// a word, in another line, that the last to arrive sets for the rest to see
+// (both zero before the launch).  With every block reading the counter, or a
+// flag of every other block, the meeting took 2.8 and 5 us for 152 to 304
+// blocks: the readers queued at one line with the arrivals.
+struct MeetPlace {
+    unsigned arrived;
+    unsigned pad0[31];
+    unsigned released;
+    unsigned pad1[31];
+};
+
+// Spins until `ready()`.  Bounded: after two seconds ST_TIMEOUT and false.
+template <typename Ready>
+__device__ __forceinline__ bool build_spin(int* status, Ready ready)
 {
-    __shared__ int s_ok;
+    uint64_t t0 = 0;
+    for (unsigned it = 1; !ready(); ++it) {
+        if ((it & 63u) != 0u) continue;
+        uint64_t t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (t0 == 0) t0 = t;
+        if (t - t0 > kBuildWaitNs) {
+            raise_status(status, ST_TIMEOUT);
+            return false;
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_release(unsigned* p, unsigned v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// The `blocks` blocks of a cooperative launch meet for the `met`-th time (this
+// counts it), what each wrote before visible to all after.  One block alone
+// only meets its own threads.  False in every thread when the wait ran out.
+__device__ bool build_meet(MeetPlace* at, unsigned blocks, unsigned& met, int* status)
+{
     __syncthreads();
     if (blocks == 1) return true;
-    ++phase;
+    ++met;
+    bool ok = true;
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(counter, 1u);
-        const unsigned target = phase * blocks;
-        uint64_t t0 = 0;
-        int ok = 1;
-        for (unsigned it = 0; *(volatile unsigned*)counter < target; ++it) {
-            if ((it & 63u) != 63u) continue;
-            uint64_t t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (t0 == 0) t0 = t;
-            if (t - t0 > kBuildWaitNs) {
-                raise_status(status, ST_TIMEOUT);
-                ok = 0;
-                break;
-            }
+        if (atomicAdd(&at->arrived, 1u) + 1u == met * blocks) {
+            __threadfence();
+            st_release(&at->released, met);
+        } else {
+            ok = build_spin(status, [&] { return ld_acquire(&at->released) >= met; });
         }
-        __threadfence();
-        s_ok = ok;
     }
-    __syncthreads();
-    return s_ok != 0;
+    return __syncthreads_and(ok) != 0;
 }
 
 // exclusive prefix of v over the block's threads, and the block's sum
@@ -411,12 +442,18 @@ __device__ __forceinline__ T block_prefix(T v, T& total)
     __syncthreads();
     if (lane == 31) s_sum[warp] = x;
     __syncthreads();
-    T before = 0, sum = 0;
+    // every warp adds up the warps' sums for itself
+    const T y = lane < kWarps ? s_sum[lane] : T(0);
+    T before = lane < warp ? y : T(0), sum = y;
+    if constexpr (sizeof(T) == 4) {
+        before = __reduce_add_sync(0xffffffffu, before);
+        sum = __reduce_add_sync(0xffffffffu, sum);
+    } else {
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const T y = s_sum[w];
-        if (w < warp) before += y;
-        sum += y;
+        for (int o = 16; o > 0; o >>= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        }
     }
     total = sum;
     return before + x - v;
@@ -424,175 +461,412 @@ __device__ __forceinline__ T block_prefix(T v, T& total)
 
 constexpr int kPlocThreads = 512;
 constexpr int kPlocMaxRadius = 64;
+constexpr int kPlocSolo = kPlocThreads;  // clusters one block finishes alone, in shared memory
+constexpr int kPlocWide = 2;             // clusters a thread takes at most
+constexpr int kPlocMaxBlocks = kPlocThreads;
+constexpr int kPlocSpan = kPlocWide * kPlocThreads + 2 * kPlocMaxRadius;
 
 struct PlocArgs {
     const float4* tris;
     int n;
     float4* cluster[2];           // [2 n] each: lo, ref bits; hi, height bits (the rounds alternate)
     int* mate;                    // [n] >= 0: merges with that later position; -1: stays; -2: merged away
-    unsigned long long* total;    // per tile: merges << 32 | clusters that stay
+    // per block: its merges << 28 | clusters that stay; and, in a sector of its
+    // own, those before it and of all, each with the round's tag << 56
+    unsigned long long* total;    // [kPlocMaxBlocks]
+    unsigned long long* answer;   // [kPlocMaxBlocks][4]
     float4* nodes;
     int* max_height;
     int radius;
     AreaW w;
-    unsigned* counter;
+    MeetPlace* place;             // the blocks' meetings and exchanges (two), zero before the launch
     int* status;
 };
 
-// The whole clustering in one cooperative launch.  A tile is kPlocThreads -
-// 2 radius clusters; its block keeps the boxes within 2 radius of it in
-// shared memory and finds the nearest neighbours of its clusters and of
-// `radius` more on either side, so that it can tell mutual pairs by itself.
-// Per round: mates and counts, a meeting of the blocks, the merges at
-// positions from the counts of the tiles before, a meeting.  With at most two
-// tiles left block 0 goes on alone and meets nobody.
-//
-// What bounds it: six kernels and a host round trip a round (63 rounds at 1M
-// triangles) left it waiting for launches; here a round's cost is its two
-// meetings and, in the first rounds, the 2 radius box unions per cluster.
-// Measured at 1M triangles: PLOC 3.3 ms -> see the note in build_ploc.
-__global__ void __launch_bounds__(kPlocThreads, 2) k_ploc(PlocArgs a)
+// Clusters in shared memory: lo x y z, hi x y z, ref bits, height bits.
+typedef float PlocShared[8][kPlocSpan];
+
+__device__ __forceinline__ void ploc_put(PlocShared& c, int k, float4 lo, float4 hi)
 {
-    __shared__ float s_box[6][kPlocThreads + 2 * kPlocMaxRadius];
-    __shared__ int s_nn[kPlocThreads];
-    const int tid = threadIdx.x, r = a.radius;
-    const int T = kPlocThreads - 2 * r;
-    unsigned blocks = gridDim.x, phase = 0;
-    for (int i = blockIdx.x * kPlocThreads + tid; i < a.n; i += gridDim.x * kPlocThreads) {
-        const Box b = leaf_box(a.tris, i);
-        __stcg(&a.cluster[0][2 * (int64_t)i], make_float4(b.lo[0], b.lo[1], b.lo[2], __int_as_float(~i)));
-        __stcg(&a.cluster[0][2 * (int64_t)i + 1], make_float4(b.hi[0], b.hi[1], b.hi[2], __int_as_float(0)));
-    }
-    if (!build_barrier(a.counter, blocks, phase, a.status)) return;
-    int nc = a.n, id_top = a.n - 2;
-    bool force = false;
-    const float4* C = a.cluster[0];
-    float4* D = a.cluster[1];
-    while (nc > 1) {
-        const int tiles = (nc + T - 1) / T;
-        if (tiles <= 2 && blocks > 1) {
-            if (blockIdx.x != 0) return;
-            blocks = 1;
-        }
-        const int per = (tiles + (int)blocks - 1) / (int)blocks;
-        const int t0 = min((int)blockIdx.x * per, tiles), t1 = min(t0 + per, tiles);
-        for (int t = t0; t < t1; ++t) {
-            const int base = t * T;
-            const int from = base - 2 * r, span = T + 4 * r;
-            for (int k = tid; k < span; k += kPlocThreads) {
-                const int e = from + k;
-                if (e < 0 || e >= nc) continue;
-                const float4 lo = __ldcg(&C[2 * (int64_t)e]), hi = __ldcg(&C[2 * (int64_t)e + 1]);
-                s_box[0][k] = lo.x; s_box[1][k] = lo.y; s_box[2][k] = lo.z;
-                s_box[3][k] = hi.x; s_box[4][k] = hi.y; s_box[5][k] = hi.z;
-            }
-            __syncthreads();
-            // thread t: cluster base - r + t, at k = r + t of the boxes
-            const int e = base - r + tid;
-            int best = -1;
-            if (e >= 0 && e < nc && !force) {
-                const int k = r + tid;
-                const float4 alo = make_float4(s_box[0][k], s_box[1][k], s_box[2][k], 0.0f);
-                const float4 ahi = make_float4(s_box[3][k], s_box[4][k], s_box[5][k], 0.0f);
-                float best_d = INFINITY;
-                const int lo = max(e - r, 0) - from, hi = min(e + r, nc - 1) - from;
+    c[0][k] = lo.x; c[1][k] = lo.y; c[2][k] = lo.z;
+    c[3][k] = hi.x; c[4][k] = hi.y; c[5][k] = hi.z;
+    c[6][k] = lo.w; c[7][k] = hi.w;
+}
+
+__device__ __forceinline__ void ploc_get(const PlocShared& c, int k, float4& lo, float4& hi)
+{
+    lo = make_float4(c[0][k], c[1][k], c[2][k], c[6][k]);
+    hi = make_float4(c[3][k], c[4][k], c[5][k], c[7][k]);
+}
+
+// Nearest neighbour of the cluster at k among those at lo..hi (all in shared
+// memory), found by `lanes` neighbouring lanes (a power of two), lane `sub` of
+// them taking its share in order; ties to the lowest.  -1: none.
+__device__ __forceinline__ int ploc_nearest(const PlocShared& c, int k, int lo, int hi, int lanes, int sub, AreaW w)
+{
+    const float4 alo = make_float4(c[0][k], c[1][k], c[2][k], 0.0f);
+    const float4 ahi = make_float4(c[3][k], c[4][k], c[5][k], 0.0f);
+    const int share = (hi - lo + lanes) / lanes;
+    const int j0 = lo + sub * share, j1 = min(j0 + share - 1, hi);
+    float best_d = INFINITY;
+    int best = -1;
 #pragma unroll 4
-                for (int j = lo; j <= hi; ++j) {
-                    const float d = union_half_area(alo, ahi, make_float4(s_box[0][j], s_box[1][j], s_box[2][j], 0.0f),
-                                                    make_float4(s_box[3][j], s_box[4][j], s_box[5][j], 0.0f), a.w);
-                    if (j != k && d < best_d) {  // ascending j: ties keep the lower position
-                        best_d = d;
-                        best = j + from;
-                    }
+    for (int j = j0; j <= j1; ++j) {
+        const float d = union_half_area(alo, ahi, make_float4(c[0][j], c[1][j], c[2][j], 0.0f),
+                                        make_float4(c[3][j], c[4][j], c[5][j], 0.0f), w);
+        if (j != k && d < best_d) {  // ascending j: ties keep the lower position
+            best_d = d;
+            best = j;
+        }
+    }
+    for (int o = 1; o < lanes; o <<= 1) {
+        const float d = __shfl_xor_sync(0xffffffffu, best_d, o);
+        const int j = __shfl_xor_sync(0xffffffffu, best, o);
+        if (d < best_d || (d == best_d && (unsigned)j < (unsigned)best)) {
+            best_d = d;
+            best = j;
+        }
+    }
+    return best;
+}
+
+// Nearest neighbours of the two clusters at k and k + 1 (k even) within `r` of
+// each: the window's boxes are read two at a time, each serving both searches.  Places outside the array hold boxes whose union with
+// anything is infinite.  best[i] is -1 for none.
+__device__ __forceinline__ void ploc_nearest2(const PlocShared& c, int k, int r, AreaW w, int best[2])
+{
+    constexpr int K = 2;
+    float al[3][K], ah[3][K];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        *(float2*)al[x] = *(const float2*)&c[x][k];
+        *(float2*)ah[x] = *(const float2*)&c[3 + x][k];
+    }
+    float best_d[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        best_d[i] = INFINITY;
+        best[i] = -1;
+    }
+    const int h = (r + K - 1) / K * K;
+    for (int g = -h; g <= h; g += K) {
+        float bl[3][K], bh[3][K];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            *(float2*)bl[x] = *(const float2*)&c[x][k + g];
+            *(float2*)bh[x] = *(const float2*)&c[3 + x][k + g];
+        }
+        // all K x K pairs within r of each other, and none a cluster with itself
+        const bool whole = g != 0 && g - (K - 1) >= -r && g + (K - 1) <= r;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const int off = g + j - i;
+                const float d = union_half_area(make_float4(al[0][i], al[1][i], al[2][i], 0.0f),
+                                                make_float4(ah[0][i], ah[1][i], ah[2][i], 0.0f),
+                                                make_float4(bl[0][j], bl[1][j], bl[2][j], 0.0f),
+                                                make_float4(bh[0][j], bh[1][j], bh[2][j], 0.0f), w);
+                // ascending position: ties keep the lower one
+                if (d < best_d[i] && (whole || (off != 0 && off >= -r && off <= r))) {
+                    best_d[i] = d;
+                    best[i] = k + g + j;
                 }
             }
-            s_nn[tid] = best;
-            __syncthreads();
-            bool stays = false, merges = false;
-            if (tid >= r && tid < r + T && e < nc) {
-                int mate = -1;
-                if (force) {
-                    // no mutual pair anywhere (not expected): positions 2k and 2k + 1 merge
-                    if (e % 2 == 1) mate = -2;
-                    else if (e + 1 < nc) mate = e + 1;
-                } else if (best >= 0 && s_nn[best - (base - r)] == e) {
-                    mate = e < best ? best : -2;
-                }
-                stays = mate != -2;
-                merges = mate >= 0;
-                __stcg(&a.mate[e], mate);
-            }
-            const int n_stay = __syncthreads_count(stays), n_merge = __syncthreads_count(merges);
-            if (tid == 0) __stcg(&a.total[t], ((unsigned long long)n_merge << 32) | (unsigned)n_stay);
         }
-        if (!build_barrier(a.counter, blocks, phase, a.status)) return;
-        // merges and stays before this block's tiles, and in all
-        unsigned long long before = 0, all = 0;
-        for (int t = tid; t < tiles; t += kPlocThreads) {
-            const unsigned long long v = __ldcg(&a.total[t]);
-            all += v;
-            if (t < t0) before += v;
-        }
-        unsigned long long sum_before, sum_all;
-        block_prefix<kPlocThreads>(before, sum_before);
-        block_prefix<kPlocThreads>(all, sum_all);
-        if ((sum_all >> 32) == 0) {
-            force = true;
-            if (!build_barrier(a.counter, blocks, phase, a.status)) return;
-            continue;
-        }
-        force = false;
-        for (int t = t0; t < t1; ++t) {
-            const int e = t * T + tid;
-            const int mate = tid < T && e < nc ? __ldcg(&a.mate[e]) : -2;
-            unsigned long long in_tile;
-            const unsigned long long at =
-                sum_before + block_prefix<kPlocThreads>(
-                                 mate == -2 ? 0ull : ((unsigned long long)(mate >= 0) << 32) | 1ull, in_tile);
-            sum_before += in_tile;
-            if (mate == -2) continue;
-            const int out = (int)(at & 0xFFFFFFFFull);
-            float4 lo = __ldcg(&C[2 * (int64_t)e]), hi = __ldcg(&C[2 * (int64_t)e + 1]);
-            if (mate >= 0) {
-                const int id = id_top - (int)(at >> 32);
-                const float4 rlo = __ldcg(&C[2 * (int64_t)mate]), rhi = __ldcg(&C[2 * (int64_t)mate + 1]);
-                a.nodes[4 * (int64_t)id + 0] = make_float4(lo.x, hi.x, lo.y, hi.y);
-                a.nodes[4 * (int64_t)id + 1] = make_float4(rlo.x, rhi.x, rlo.y, rhi.y);
-                a.nodes[4 * (int64_t)id + 2] = make_float4(lo.z, hi.z, rlo.z, rhi.z);
-                a.nodes[4 * (int64_t)id + 3] = make_float4(lo.w, rlo.w, 0.0f, 0.0f);
-                const int h = 1 + max(__float_as_int(hi.w), __float_as_int(rhi.w));
-                lo = make_float4(fminf(lo.x, rlo.x), fminf(lo.y, rlo.y), fminf(lo.z, rlo.z), __int_as_float(id));
-                hi = make_float4(fmaxf(hi.x, rhi.x), fmaxf(hi.y, rhi.y), fmaxf(hi.z, rhi.z), __int_as_float(h));
-                if (id == 0) *a.max_height = h;
-            }
-            __stcg(&D[2 * (int64_t)out], lo);
-            __stcg(&D[2 * (int64_t)out + 1], hi);
-        }
-        id_top -= (int)(sum_all >> 32);
-        nc = (int)(sum_all & 0xFFFFFFFFull);
-        const float4* swap = C;
-        C = D;
-        D = const_cast<float4*>(swap);
-        if (!build_barrier(a.counter, blocks, phase, a.status)) return;
     }
 }
 
+// What position e of nc does, given its and its neighbour's nearest.
+__device__ __forceinline__ int ploc_mate(int e, int nc, int best, int best_of_best, bool force)
+{
+    if (force) return e % 2 == 1 ? -2 : (e + 1 < nc ? e + 1 : -1);  // no mutual pair anywhere (not expected)
+    if (best < 0 || best_of_best != e) return -1;
+    return e < best ? best : -2;
+}
+
+// Merges the cluster (rlo, rhi) into (lo, hi) as node `id`.
+__device__ __forceinline__ void ploc_merge(const PlocArgs& a, int id, float4& lo, float4& hi, float4 rlo, float4 rhi)
+{
+    a.nodes[4 * (int64_t)id + 0] = make_float4(lo.x, hi.x, lo.y, hi.y);
+    a.nodes[4 * (int64_t)id + 1] = make_float4(rlo.x, rhi.x, rlo.y, rhi.y);
+    a.nodes[4 * (int64_t)id + 2] = make_float4(lo.z, hi.z, rlo.z, rhi.z);
+    a.nodes[4 * (int64_t)id + 3] = make_float4(lo.w, rlo.w, 0.0f, 0.0f);
+    const int h = 1 + max(__float_as_int(hi.w), __float_as_int(rhi.w));
+    lo = make_float4(fminf(lo.x, rlo.x), fminf(lo.y, rlo.y), fminf(lo.z, rlo.z), __int_as_float(id));
+    hi = make_float4(fmaxf(hi.x, rhi.x), fmaxf(hi.y, rhi.y), fmaxf(hi.z, rhi.z), __int_as_float(h));
+    if (id == 0) *a.max_height = h;
+}
+
+// The rounds from kPlocSolo clusters on, by one block out of shared memory.
+__device__ void ploc_solo(const PlocArgs& a, const float4* C, int nc, int id_top, PlocShared& c, int* s_nn)
+{
+    const int tid = threadIdx.x, r = a.radius;
+    __syncthreads();
+    for (int k = tid; k < nc; k += kPlocThreads) ploc_put(c, k, __ldcg(&C[2 * (int64_t)k]), __ldcg(&C[2 * (int64_t)k + 1]));
+    __syncthreads();
+    bool force = false;
+    while (nc > 1) {
+        int lanes = 1;
+        while (lanes < 32 && 2 * lanes * nc <= kPlocThreads) lanes *= 2;
+        {
+            const int e = tid / lanes, k = min(e, nc - 1);
+            const int best = force ? -1 : ploc_nearest(c, k, max(k - r, 0), min(k + r, nc - 1), lanes, tid % lanes, a.w);
+            if (e < nc && tid % lanes == 0) s_nn[e] = best;
+        }
+        __syncthreads();
+        int mate = -2;
+        float4 lo, hi, rlo, rhi;
+        if (tid < nc) {
+            const int best = s_nn[tid];
+            mate = ploc_mate(tid, nc, best, best >= 0 ? s_nn[best] : -1, force);
+            if (mate != -2) ploc_get(c, tid, lo, hi);
+            if (mate >= 0) ploc_get(c, mate, rlo, rhi);
+        }
+        unsigned sum;
+        const unsigned at =  // (its barriers end the reads)
+            block_prefix<kPlocThreads>(mate == -2 ? 0u : (mate >= 0 ? 0x10001u : 1u), sum);
+        force = (sum >> 16) == 0;
+        if (force) continue;
+        if (mate != -2) {
+            if (mate >= 0) ploc_merge(a, id_top - (int)(at >> 16), lo, hi, rlo, rhi);
+            ploc_put(c, (int)(at & 0xFFFFu), lo, hi);
+        }
+        id_top -= (int)(sum >> 16);
+        nc = (int)(sum & 0xFFFFu);
+        __syncthreads();
+    }
+}
+
+// One round of the blocks' clustering.  A tile is what a block's threads
+// hold, K clusters each or one per `lanes` threads, less `halo` on either
+// side: the block keeps the boxes within twice the halo in shared memory and
+// finds the nearest neighbours of the halo's clusters too, so that it can tell
+// mutual pairs by itself.  The blocks then exchange their counts and write the
+// merged array at the positions those give.
+struct PlocRound {
+    const float4* C;
+    float4* D;
+    int nc, id_top, lanes;
+    bool force;
+    unsigned round;
+};
+
+template <int K>
+__device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, int* s_nn, unsigned blocks, const PlocRound& g,
+                           unsigned long long& all)
+{
+    __shared__ unsigned long long s_sum[2];
+    const int tid = threadIdx.x, r = a.radius, nc = g.nc;
+    const int lanes = K > 1 ? 1 : g.lanes;
+    const int halo = K > 1 ? (r + 1) & ~1 : r;
+    const int E = K > 1 ? K * kPlocThreads : kPlocThreads / lanes;  // clusters held, T of them the tile's own
+    const int T = E - 2 * halo;
+    const int tiles = (nc + T - 1) / T;
+    const int per = (tiles + (int)blocks - 1) / (int)blocks;
+    const int t0 = min((int)blockIdx.x * per, tiles), t1 = min(t0 + per, tiles);
+    const int first = K > 1 ? K * tid : tid / lanes;  // this thread's first cluster of those held
+    int mate[K];                                      // of the last tile's
+    unsigned place = 0, count;                        // merges << 16 | stays before this thread's, and of the tile
+    unsigned long long mine = 0;                      // merges << 32 | stays of the block's tiles
+#pragma unroll
+    for (int i = 0; i < K; ++i) mate[i] = -2;
+    for (int t = t0; t < t1; ++t) {
+        const int base = t * T, from = base - 2 * halo, span = T + 4 * halo;
+        for (int k = tid; k < span; k += kPlocThreads) {
+            const int e = from + k;
+            if (e >= 0 && e < nc) {
+                ploc_put(s_c, k, __ldcg(&g.C[2 * (int64_t)e]), __ldcg(&g.C[2 * (int64_t)e + 1]));
+            } else if (K > 1) {
+                ploc_put(s_c, k, make_float4(-INFINITY, -INFINITY, -INFINITY, 0.0f),
+                         make_float4(INFINITY, INFINITY, INFINITY, 0.0f));
+            }
+        }
+        __syncthreads();
+        // held cluster m is e = base - halo + m, at halo + m of the boxes
+        if constexpr (K > 1) {
+            int best[K];
+#pragma unroll
+            for (int i = 0; i < K; ++i) best[i] = -1;
+            if (!g.force) ploc_nearest2(s_c, halo + first, r, a.w, best);
+            *(int2*)&s_nn[first] = make_int2(best[0], best[1]);
+        } else {
+            const int e = min(max(base - halo + first, 0), nc - 1);
+            int best = -1;
+            if (!g.force)
+                best = ploc_nearest(s_c, e - from, max(e - r, 0) - from, min(e + r, nc - 1) - from, lanes, tid % lanes,
+                                    a.w);
+            if (tid % lanes == 0) s_nn[first] = best;
+        }
+        __syncthreads();
+        unsigned v = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const int m = first + i, e = base - halo + m;
+            mate[i] = -2;
+            if (tid % lanes != 0 || m < halo || m >= halo + T || e >= nc) continue;
+            const int best = s_nn[m];
+            mate[i] = ploc_mate(e, nc, best < 0 ? -1 : best + from, best < 0 ? -1 : s_nn[best - halo] + from, g.force);
+            if (per > 1) __stcg(&a.mate[e], mate[i]);
+            if (mate[i] != -2) v += mate[i] >= 0 ? 0x10001u : 1u;
+        }
+        place = block_prefix<kPlocThreads>(v, count);
+        mine += ((unsigned long long)(count >> 16) << 32) | (count & 0xFFFFu);
+    }
+    // merges and stays of the blocks before, and of all
+    unsigned long long before = 0;
+    all = mine;
+    if (blocks > 1) {
+        // every block leaves its counts and arrives; the last one sums them up
+        // and answers each in its own sector
+        const unsigned long long tag = (unsigned long long)(g.round % 200u + 1u) << 56;
+        MeetPlace* at = a.place + 1;
+        bool last = false;
+        if (tid == 0) {
+            __stcg(&a.total[blockIdx.x], ((mine >> 32) << 28) | (mine & 0xFFFFFFFull));
+            __threadfence();
+            last = atomicAdd(&at->arrived, 1u) + 1u == (g.round + 1u) * blocks;
+        }
+        if (__syncthreads_or(last)) {
+            __threadfence();
+            const unsigned long long v = tid < (int)blocks ? __ldcg(&a.total[tid]) : 0ull;
+            unsigned long long sum;
+            const unsigned long long x = block_prefix<kPlocThreads>(v, sum);
+            if (tid < (int)blocks) {
+                *(volatile unsigned long long*)&a.answer[4 * tid] = tag | x;
+                *(volatile unsigned long long*)&a.answer[4 * tid + 1] = tag | sum;
+            }
+        }
+        bool ok = true;
+        if (tid == 0) {
+            const volatile unsigned long long* mine_at = a.answer + 4 * blockIdx.x;
+            unsigned long long x = 0, y = 0;
+            ok = build_spin(a.status, [&] {
+                x = mine_at[0];
+                y = mine_at[1];
+                return (x >> 56) == (tag >> 56) && (y >> 56) == (tag >> 56);
+            });
+            s_sum[0] = x;
+            s_sum[1] = y;
+        }
+        if (!__syncthreads_and(ok)) return false;
+        before = ((s_sum[0] >> 28 & 0xFFFFFFFull) << 32) | (s_sum[0] & 0xFFFFFFFull);
+        all = ((s_sum[1] >> 28 & 0xFFFFFFFull) << 32) | (s_sum[1] & 0xFFFFFFFull);
+    }
+    if ((all >> 32) == 0) return true;
+    // the tile at `base`, its boxes in shared memory and its mates in registers
+    auto write = [&](int base, unsigned long long at) {
+        const int from = base - 2 * halo;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            if (mate[i] == -2) continue;
+            float4 lo, hi;
+            ploc_get(s_c, halo + first + i, lo, hi);
+            if (mate[i] >= 0) {
+                float4 rlo, rhi;
+                ploc_get(s_c, mate[i] - from, rlo, rhi);
+                ploc_merge(a, g.id_top - (int)(at >> 32), lo, hi, rlo, rhi);
+            }
+            const int64_t out = (int64_t)(at & 0xFFFFFFFFull);
+            __stcg(&g.D[2 * out], lo);
+            __stcg(&g.D[2 * out + 1], hi);
+            at += mate[i] >= 0 ? (1ull << 32) | 1ull : 1ull;
+        }
+    };
+    auto wide = [](unsigned v) { return ((unsigned long long)(v >> 16) << 32) | (v & 0xFFFFu); };
+    if (per == 1) {
+        write(t0 * T, before + wide(place));
+        return true;
+    }
+    for (int t = t0; t < t1; ++t) {
+        const int base = t * T, from = base - 2 * halo;
+        for (int k = 2 * halo + tid; k < T + 3 * halo; k += kPlocThreads)
+            if (from + k < nc)
+                ploc_put(s_c, k, __ldcg(&g.C[2 * (int64_t)(from + k)]), __ldcg(&g.C[2 * (int64_t)(from + k) + 1]));
+        unsigned v = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const int m = first + i, e = base - halo + m;
+            mate[i] = m >= halo && m < halo + T && e < nc ? __ldcg(&a.mate[e]) : -2;
+            if (mate[i] != -2) v += mate[i] >= 0 ? 0x10001u : 1u;
+        }
+        const unsigned p = block_prefix<kPlocThreads>(v, count);  // (its barriers end the loads)
+        write(base, before + wide(p));
+        before += wide(count);
+        __syncthreads();
+    }
+    return true;
+}
+
+constexpr size_t kPlocShared = sizeof(PlocShared) + kPlocWide * kPlocThreads * sizeof(int);
+
+// The whole clustering in one cooperative launch, a round at a time: two
+// clusters a thread while the blocks' threads are fewer than the clusters,
+// then one, then one per 2, 4 or 8 lanes; the last kPlocSolo of them block 0
+// finishes alone, meeting nobody.
+//
+// What bounds it: six kernels and a host round trip a round (63 rounds at 1M
+// triangles, 3.3 ms) left it waiting for launches.  In one launch it is a
+// round's chain (an exchange of counts and a meeting, ~5 us, a search) and, in
+// the first rounds, the 2 radius box unions per cluster (~30 issue slots each,
+// half of them min / max).  1M triangles: 0.69 ms with one cluster a thread,
+// everything through L2 and the blocks polling one counter; 0.58 ms so.  Four
+// clusters a thread, or 1,024 threads, take as long: the searches are bound
+// by issue, the rest by the chain.
+__global__ void __launch_bounds__(kPlocThreads, 1) k_ploc(PlocArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    PlocShared& s_c = *(PlocShared*)smem;
+    int* s_nn = (int*)(smem + sizeof(PlocShared));
+    const int r = a.radius;
+    const unsigned blocks = gridDim.x;
+    unsigned met = 0;
+    for (int64_t i = blockIdx.x * kPlocThreads + threadIdx.x; i < a.n; i += gridDim.x * kPlocThreads) {
+        const Box b = leaf_box(a.tris, (int)i);
+        __stcg(&a.cluster[0][2 * i], make_float4(b.lo[0], b.lo[1], b.lo[2], __int_as_float(~(int)i)));
+        __stcg(&a.cluster[0][2 * i + 1], make_float4(b.hi[0], b.hi[1], b.hi[2], __int_as_float(0)));
+    }
+    if (!build_meet(a.place, blocks, met, a.status)) return;
+    PlocRound g{a.cluster[0], a.cluster[1], a.n, a.n - 2, 1, false, 0};
+    while (g.nc > kPlocSolo) {
+        // the most lanes a cluster with which every block still has one tile at most
+        g.lanes = 0;
+        for (int l = 8; l >= 1 && g.lanes == 0; l >>= 1) {
+            const int T = kPlocThreads / l - 2 * r;
+            if (T >= 32 && (int64_t)T * blocks >= g.nc) g.lanes = l;
+        }
+        unsigned long long all;
+        if (!(g.lanes ? ploc_round<1>(a, s_c, s_nn, blocks, g, all) : ploc_round<kPlocWide>(a, s_c, s_nn, blocks, g, all)))
+            return;
+        ++g.round;
+        g.force = (all >> 32) == 0;  // then nothing was written
+        if (!g.force) {
+            g.id_top -= (int)(all >> 32);
+            g.nc = (int)(all & 0xFFFFFFFFull);
+            const float4* swap = g.C;
+            g.C = g.D;
+            g.D = const_cast<float4*>(swap);
+        }
+        if (!build_meet(a.place, blocks, met, a.status)) return;
+    }
+    if (blockIdx.x == 0) ploc_solo(a, g.C, g.nc, g.id_top, s_c, s_nn);
+}
+
 // blocks of a cooperative launch of `fn`, at most `want`; 1 without cooperative launch
-int coop_blocks(const void* fn, int threads, int num_sms, int coop, int64_t want)
+int coop_blocks(const void* fn, int threads, size_t smem, int num_sms, int coop, int64_t want)
 {
     int per_sm = 0;
-    if (!coop || want <= 1 || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0) != cudaSuccess)
+    if (!coop || want <= 1 || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess)
         return 1;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)per_sm * num_sms));
+    return (int)std::max<int64_t>(1, std::min(want, (int64_t)per_sm * num_sms));
 }
 
 }  // namespace
 
 size_t ploc_scratch_bytes(int64_t n)
 {
-    const size_t tiles = (size_t)(n + kPlocThreads - 2 * kPlocMaxRadius - 1) / (kPlocThreads - 2 * kPlocMaxRadius);
     return 2 * align256((size_t)n * 2 * sizeof(float4)) + align256(n * sizeof(int)) +
-           align256(tiles * sizeof(unsigned long long)) + 256;
+           align256(2 * sizeof(MeetPlace)) + kPlocMaxBlocks * 5 * sizeof(unsigned long long);
 }
 
 cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, float4* nodes_out, int* max_height_dev,
@@ -600,7 +874,6 @@ cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, flo
 {
     if (n < 2 || radius < 1 || radius > kPlocMaxRadius) return cudaErrorInvalidValue;
     if (scratch_bytes < ploc_scratch_bytes(n)) return cudaErrorInvalidValue;
-    const size_t tiles = (size_t)(n + kPlocThreads - 2 * kPlocMaxRadius - 1) / (kPlocThreads - 2 * kPlocMaxRadius);
     char* p = (char*)scratch;
     PlocArgs a;
     a.tris = tris_sorted;
@@ -610,24 +883,27 @@ cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, flo
         p += align256((size_t)n * 2 * sizeof(float4));
     }
     a.mate = (int*)p; p += align256(n * sizeof(int));
-    a.total = (unsigned long long*)p; p += align256(tiles * sizeof(unsigned long long));
+    char* zero = p;
+    a.place = (MeetPlace*)p; p += align256(2 * sizeof(MeetPlace));
+    a.answer = (unsigned long long*)p; p += kPlocMaxBlocks * 4 * sizeof(unsigned long long);
+    a.total = (unsigned long long*)p; p += kPlocMaxBlocks * sizeof(unsigned long long);
     a.nodes = nodes_out;
     a.max_height = max_height_dev;
     a.radius = radius;
     a.w = w;
-    a.counter = (unsigned*)p;
     a.status = status;
-    cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned), s);
+    cudaError_t e = cudaMemsetAsync(zero, 0, (size_t)(p - zero), s);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_ploc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlocShared);
     if (e != cudaSuccess) return e;
-    const int T = kPlocThreads - 2 * radius;
-    const int64_t want = (n + T - 1) / T;
-    const int grid = coop_blocks((const void*)k_ploc, kPlocThreads, num_sms, coop, want <= 2 ? 1 : want);
+    const int grid = coop_blocks((const void*)k_ploc, kPlocThreads, kPlocShared, num_sms, coop,
+                                 n <= kPlocSolo ? 1 : std::min<int64_t>((n + 31) / 32, kPlocMaxBlocks));
     if (grid == 1) {
-        k_ploc<<<1, kPlocThreads, 0, s>>>(a);
+        k_ploc<<<1, kPlocThreads, kPlocShared, s>>>(a);
         return cudaGetLastError();
     }
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void*)k_ploc, dim3(grid), dim3(kPlocThreads), args, 0, s);
+    return cudaLaunchCooperativeKernel((const void*)k_ploc, dim3(grid), dim3(kPlocThreads), args, kPlocShared, s);
 }
 
 }  // namespace lidar
@@ -861,7 +1137,7 @@ struct CollapseTree {
     int* kids;            // [level][W] internal children of the level being walked
     unsigned* total;      // per tile of a level: internal children
     int* state;           // the lone first block's level: nodes, first slot, levels
-    unsigned* counter;    // the meetings of this tree's blocks, zero before the launch
+    MeetPlace* place;     // the meetings of this tree's blocks, zero before the launch
     WideInfo* info;       // stack_need zero before the launch
 };
 
@@ -877,7 +1153,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
 {
     constexpr int T = kCollapseThreads;
     const int tid = threadIdx.x;
-    unsigned phase = 0;
+    unsigned met = 0;
     int n = 1, base = 0, levels = 0, need = 0;
     // one level by blocks `me` of `of`: false when a meeting ran out
     auto level = [&](unsigned me, unsigned of) -> bool {
@@ -902,7 +1178,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
             block_prefix<T>((unsigned)internal, sum);
             if (tid == 0) __stcg(&c.total[t], sum);
         }
-        if (!build_barrier(c.counter, of, phase, a.status)) return false;
+        if (!build_meet(c.place, of, met, a.status)) return false;
         unsigned before = 0, all = 0;
         for (int t = tid; t < tiles; t += T) {
             const unsigned v = __ldcg(&c.total[t]);
@@ -929,7 +1205,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
         base += n;
         n = (int)next;
         ++levels;
-        return build_barrier(c.counter, of, phase, a.status);
+        return build_meet(c.place, of, met, a.status);
     };
     // the first levels fit one block, which walks them alone while the others wait once
     if (blocks > 1) {
@@ -941,7 +1217,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
                 __stcg(&c.state[2], levels);
             }
         }
-        if (!build_barrier(c.counter, blocks, phase, a.status)) return;
+        if (!build_meet(c.place, blocks, met, a.status)) return;
         n = __ldcg(&c.state[0]);
         base = __ldcg(&c.state[1]);
         levels = __ldcg(&c.state[2]);
@@ -1033,7 +1309,7 @@ namespace {
 // layout of the collapse's scratch (`base` may be NULL to size it)
 struct CollapseScratch {
     CollapseArgs a{};
-    unsigned* counters;
+    MeetPlace* places;
     int *parent_node, *parent_leaf;
     size_t bytes;
 
@@ -1048,11 +1324,11 @@ struct CollapseScratch {
             at += (b + 255) / 256 * 256;
             return p;
         };
-        counters = (unsigned*)get(2 * sizeof(unsigned) + 8 * sizeof(int));
+        places = (MeetPlace*)get(2 * sizeof(MeetPlace) + 8 * sizeof(int));
         for (int k = 0; k < 2; ++k) {
             CollapseTree& t = a.tree[k];
-            t.counter = counters + k;
-            t.state = (int*)(counters + 2) + 4 * k;
+            t.place = places + k;
+            t.state = (int*)(places + 2) + 4 * k;
             t.root = (int*)get(m * sizeof(int));
             t.first = (int*)get(m * sizeof(int));
             t.pushes = (int*)get(m * sizeof(int));
@@ -1107,7 +1383,7 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
     }
     c.a.tree[0].info = info_dev;
     c.a.tree[1].info = info_dev + 1;
-    cudaError_t e = cudaMemsetAsync(c.counters, 0, 2 * sizeof(unsigned), s);
+    cudaError_t e = cudaMemsetAsync(c.places, 0, 2 * sizeof(MeetPlace), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(info_dev, 0, 2 * sizeof(WideInfo), s);
     if (e != cudaSuccess) return e;
     if (sah_dp) {
@@ -1128,7 +1404,7 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
     // two blocks (one a tree, which meet nobody) for what one block's tiles hold
     const int64_t want = 2 * ((n_binary / 4 + kCollapseThreads - 1) / kCollapseThreads);
     const int grid =
-        std::max(2, coop_blocks((const void*)k_collapse_levels, kCollapseThreads, num_sms, coop, want) / 2 * 2);
+        std::max(2, coop_blocks((const void*)k_collapse_levels, kCollapseThreads, 0, num_sms, coop, want) / 2 * 2);
     if (grid == 2) {
         k_collapse_levels<<<2, kCollapseThreads, 0, s>>>(c.a);
         e = cudaGetLastError();
