@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include "philox.cuh"
 #include "trace.cuh"
@@ -242,6 +243,10 @@ __device__ bool grid_barrier(unsigned* counter, unsigned k, int* status, uint64_
     return s_ok != 0;
 }
 
+// the 4-wide walk of a node array too large for 32-bit offsets (the launch
+// configuration's 2 stands for both)
+constexpr int kTravFar4 = 4;
+
 template <bool kCount, int kMinBlocks, int kTrav>
 __global__ void __launch_bounds__(256, kMinBlocks) k_cast(SceneDev S, const SensorDev* __restrict__ sensors,
                                               const FrameDev* __restrict__ frames, int n_frames,
@@ -271,7 +276,9 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_cast(SceneDev S, const Sens
         if (kTrav == 3)
             return trace_closest8<kCount>(S, p, t_max, h, &wc, sh_stack + threadIdx.x, blockDim.x, cost);
         if (kTrav == 2)
-            return trace_closest4<kCount>(S, p, t_max, h, &wc, sh_stack + threadIdx.x, blockDim.x, cost);
+            return trace_closest4<false, kCount>(S, p, t_max, h, &wc, sh_stack + threadIdx.x, blockDim.x, cost);
+        if (kTrav == kTravFar4)
+            return trace_closest4<true, kCount>(S, p, t_max, h, &wc, sh_stack + threadIdx.x, blockDim.x, cost);
         return trace_closest<kCount>(S, p, t_max, h, &wc, sh_stack + threadIdx.x, blockDim.x, cost);
     };
     while (true) {
@@ -641,28 +648,32 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
     const size_t stack_bytes = (size_t)kSharedStack * cfg.block_threads * sizeof(int2);
     const int bt = cfg.block_threads;
     cudaError_t e;
+    // (the bounds-checked build walks with 64-bit addresses throughout)
+    const bool far4 = kBoundsChecks || scene.n_nodes4 > kNearNodes4;
+    const int trav = cfg.traversal == 2 && far4 ? kTravFar4 : cfg.traversal;
+    auto by_residency = [&](auto w, size_t smem) {
+        constexpr int W = decltype(w)::value;
+        return variant == 2   ? launch_one<false, 2, W>(s, a, grid, bt, smem, num_sms, refused)
+               : variant == 3 ? launch_one<false, 3, W>(s, a, grid, bt, smem, num_sms, refused)
+                              : launch_one<false, 4, W>(s, a, grid, bt, smem, num_sms, refused);
+    };
     if (count) {
         // the work counted depends on the tree the traversal walks, not on the launch shape
         a.fused = 0;
-        e = cfg.traversal == 3   ? launch_one<true, 4, 3>(s, a, grid, bt, stack_bytes, num_sms, refused)
-            : cfg.traversal == 2 ? launch_one<true, 4, 2>(s, a, grid, bt, stack_bytes, num_sms, refused)
-                                 : launch_one<true, 4, 0>(s, a, grid, bt, stack_bytes, num_sms, refused);
-    } else if (cfg.traversal == 1) {
-        e = variant == 2   ? launch_one<false, 2, 1>(s, a, grid, bt, 0, num_sms, refused)
-            : variant == 3 ? launch_one<false, 3, 1>(s, a, grid, bt, 0, num_sms, refused)
-                           : launch_one<false, 4, 1>(s, a, grid, bt, 0, num_sms, refused);
-    } else if (cfg.traversal == 2) {
-        e = variant == 2   ? launch_one<false, 2, 2>(s, a, grid, bt, stack_bytes, num_sms, refused)
-            : variant == 3 ? launch_one<false, 3, 2>(s, a, grid, bt, stack_bytes, num_sms, refused)
-                           : launch_one<false, 4, 2>(s, a, grid, bt, stack_bytes, num_sms, refused);
-    } else if (cfg.traversal == 3) {
-        e = variant == 2   ? launch_one<false, 2, 3>(s, a, grid, bt, stack_bytes, num_sms, refused)
-            : variant == 3 ? launch_one<false, 3, 3>(s, a, grid, bt, stack_bytes, num_sms, refused)
-                           : launch_one<false, 4, 3>(s, a, grid, bt, stack_bytes, num_sms, refused);
+        e = trav == 3           ? launch_one<true, 4, 3>(s, a, grid, bt, stack_bytes, num_sms, refused)
+            : trav == 2         ? launch_one<true, 4, 2>(s, a, grid, bt, stack_bytes, num_sms, refused)
+            : trav == kTravFar4 ? launch_one<true, 4, kTravFar4>(s, a, grid, bt, stack_bytes, num_sms, refused)
+                                : launch_one<true, 4, 0>(s, a, grid, bt, stack_bytes, num_sms, refused);
+    } else if (trav == 1) {
+        e = by_residency(std::integral_constant<int, 1>(), 0);
+    } else if (trav == 2) {
+        e = by_residency(std::integral_constant<int, 2>(), stack_bytes);
+    } else if (trav == kTravFar4) {
+        e = by_residency(std::integral_constant<int, kTravFar4>(), stack_bytes);
+    } else if (trav == 3) {
+        e = by_residency(std::integral_constant<int, 3>(), stack_bytes);
     } else {
-        e = variant == 2   ? launch_one<false, 2, 0>(s, a, grid, bt, stack_bytes, num_sms, refused)
-            : variant == 3 ? launch_one<false, 3, 0>(s, a, grid, bt, stack_bytes, num_sms, refused)
-                           : launch_one<false, 4, 0>(s, a, grid, bt, stack_bytes, num_sms, refused);
+        e = by_residency(std::integral_constant<int, 0>(), stack_bytes);
     }
     if (e == cudaSuccess && scattered) *scattered = a.fused != 0;
     return e;

@@ -97,7 +97,7 @@ __device__ __forceinline__ void write_echoes(const EchoOut& echo, int64_t g, int
 // sweep's ray order from the work counter, as the frame cast does, so the
 // sensor's ray order and cost schedule apply.  Dense records (the strongest
 // return) and, with kEcho, the echoes of each beam's sub-rays.
-template <int kMinBlocks, bool kEcho>
+template <int kMinBlocks, bool kEcho, bool kFar>
 __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, const SensorDev* __restrict__ sensors,
                                                                  const SweepDev* __restrict__ frames, int n_frames,
                                                                  const int64_t* __restrict__ tile_prefix,
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
                 if (k > 0) subray_dir(r.dx, r.dy, r.dz, sd.alpha[k], sd.beta[k]);
                 const RayPre p = prepare_ray(r);
                 HitRec h;
-                if (active && !trace_closest4<false>(S, p, sd.t_max, h, nullptr, nullptr, 0))
+                if (active && !trace_closest4<kFar>(S, p, sd.t_max, h, nullptr, nullptr, 0))
                     raise_status(status, h.leaf == kBadIndex ? ST_BOUNDS : ST_STACK);
                 BeamResult res;
                 res.valid = 0;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
                 if (k > 0) subray_dir(r.dx, r.dy, r.dz, sd.alpha[k], sd.beta[k]);
                 const RayPre p = prepare_ray(r);
                 HitRec h;
-                if (!trace_closest4<false>(S, p, sd.t_max, h, nullptr, nullptr, 0))
+                if (!trace_closest4<kFar>(S, p, sd.t_max, h, nullptr, nullptr, 0))
                     raise_status(status, h.leaf == kBadIndex ? ST_BOUNDS : ST_STACK);
                 BeamResult res;
                 shade(S, h, r, sd, T, seed, beam, (uint32_t)f.frame, (uint32_t)f.sensor, (uint32_t)k, res);
@@ -244,9 +244,12 @@ cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDe
     const int resident = cfg.block_threads * cfg.blocks_per_sm;
     const int bt = cfg.block_threads;
     const dim3 gd((unsigned)grid);
+    // node arrays too large for 32-bit offsets (and the bounds-checked build)
+    const bool far4 = kBoundsChecks || S.n_nodes4 > kNearNodes4;
 #define LIDAR_SWEEP_LAUNCH(MB, EC)                                                                              \
-    k_sweep_tiles<MB, EC><<<gd, bt, 0, s>>>(S, sensors_dev, frames_dev, n_frames, tile_prefix_dev, n_tiles,     \
-                                            cfg.tile_rays, T, seed, out, echo, status, work_counter)
+    (far4 ? k_sweep_tiles<MB, EC, true> : k_sweep_tiles<MB, EC, false>)<<<gd, bt, 0, s>>>(                      \
+        S, sensors_dev, frames_dev, n_frames, tile_prefix_dev, n_tiles, cfg.tile_rays, T, seed, out, echo,      \
+        status, work_counter)
     const bool ec = echo.n_echoes > 0;
     if (resident <= 512) {
         if (ec) LIDAR_SWEEP_LAUNCH(2, true); else LIDAR_SWEEP_LAUNCH(2, false);

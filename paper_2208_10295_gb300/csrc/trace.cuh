@@ -322,23 +322,52 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
 
-__device__ __forceinline__ unsigned long long slab2(unsigned long long planes, unsigned long long o2,
-                                                    unsigned long long inv2)
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
 {
-    unsigned long long d, t;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(planes), "l"(o2));
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(d), "l"(inv2));
-    return t;
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// A ray's constants for the slab distances of the wide nodes: plane P of an
+// axis is met at P inv + c, one fused operation, with c = -o inv moved against
+// its rounding: by 2^-22 |o inv| (the product, the sum and the fused result
+// are each off by at most 2^-24 |o inv| more than a relative 2^-24), and by
+// 2^-20 |inv| so that a ray that lies in a plane (inv infinite: kept to
+// 1e18, where every distance the slack does not cover is beyond any range) finds itself inside the slab.
+// An entry is then never late and an exit never early, but for the relative
+// errors that kFarScale covers.  (A subtraction and a product per plane, each
+// rounded, were as conservative with twice the instructions.)
+struct SlabRay {
+    unsigned long long inv[3], near[3], far[3];  // each twice, for two planes at a time
+    int flip[3];                                 // 1: the direction is negative, the upper plane comes first
+};
+
+__device__ __forceinline__ SlabRay slab_ray(const RayPre& p)
+{
+    SlabRay s;
+    const float o[3] = {p.ox, p.oy, p.oz}, i[3] = {p.ix, p.iy, p.iz};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float inv = fminf(fmaxf(i[k], -1e18f), 1e18f);
+        const float a = o[k] * inv;
+        const float e = fmaf(fabsf(a), 2.384185791015625e-07f, fabsf(inv) * 9.5367431640625e-07f);
+        s.inv[k] = pack2(inv, inv);
+        s.near[k] = pack2(-a - e, -a - e);
+        s.far[k] = pack2(e - a, e - a);
+        s.flip[k] = inv < 0.0f ? 1 : 0;
+    }
+    return s;
 }
 
 // entry/exit planes already chosen by the ray's direction signs
-__device__ __forceinline__ void slab4_planes(float4 e, float4 x, unsigned long long o2, unsigned long long i2,
-                                             float4& tin, float4& tout)
+__device__ __forceinline__ void slab4_planes(float4 e, float4 x, unsigned long long inv, unsigned long long near,
+                                             unsigned long long far, float4& tin, float4& tout)
 {
-    unpack2(slab2(pack2(e.x, e.y), o2, i2), tin.x, tin.y);
-    unpack2(slab2(pack2(e.z, e.w), o2, i2), tin.z, tin.w);
-    unpack2(slab2(pack2(x.x, x.y), o2, i2), tout.x, tout.y);
-    unpack2(slab2(pack2(x.z, x.w), o2, i2), tout.z, tout.w);
+    unpack2(fma2(pack2(e.x, e.y), inv, near), tin.x, tin.y);
+    unpack2(fma2(pack2(e.z, e.w), inv, near), tin.z, tin.w);
+    unpack2(fma2(pack2(x.x, x.y), inv, far), tout.x, tout.y);
+    unpack2(fma2(pack2(x.z, x.w), inv, far), tout.z, tout.w);
 }
 
 // Three-input FP32 max / min (sm_100+): the same result as the two-input
@@ -360,17 +389,14 @@ __device__ __forceinline__ float min3f(float a, float b, float c)
 
 // Near and far slab distances of four child boxes (entry and exit planes per
 // axis already chosen by the direction signs): near = max(axis entries,
-// t_eps), far = min(axis exits) * kFarScale, each slab distance rounded as
-// slab_t rounds it.
+// t_eps), far = min(axis exits) * kFarScale.
 __device__ __forceinline__ void near_far4(float4 xe, float4 xx, float4 ye, float4 yx, float4 ze, float4 zx,
-                                          unsigned long long ox2, unsigned long long oy2, unsigned long long oz2,
-                                          unsigned long long ix2, unsigned long long iy2, unsigned long long iz2,
-                                          float4& kn, float4& kf)
+                                          const SlabRay& s, float4& kn, float4& kf)
 {
     float4 xi, xo, yi, yo, zi, zo;
-    slab4_planes(xe, xx, ox2, ix2, xi, xo);
-    slab4_planes(ye, yx, oy2, iy2, yi, yo);
-    slab4_planes(ze, zx, oz2, iz2, zi, zo);
+    slab4_planes(xe, xx, s.inv[0], s.near[0], s.far[0], xi, xo);
+    slab4_planes(ye, yx, s.inv[1], s.near[1], s.far[1], yi, yo);
+    slab4_planes(ze, zx, s.inv[2], s.near[2], s.far[2], zi, zo);
     kn = make_float4(max3f(xi.x, yi.x, fmaxf(zi.x, kTEps)), max3f(xi.y, yi.y, fmaxf(zi.y, kTEps)),
                      max3f(xi.z, yi.z, fmaxf(zi.z, kTEps)), max3f(xi.w, yi.w, fmaxf(zi.w, kTEps)));
     kf = make_float4(min3f(xo.x, yo.x, zo.x) * kFarScale, min3f(xo.y, yo.y, zo.y) * kFarScale,
@@ -402,7 +428,16 @@ __device__ __forceinline__ void sort2u(unsigned& a, unsigned& b)
 // to far by a 4-key sorting network over 32-bit keys (the entry distance's
 // bits with the low bits replaced by the slot, as in trace_closest8); the
 // nearest is visited next and the others pushed far-first.
-template <bool kCount = false>
+//
+// Node records are addressed as a 32-bit byte offset from the array (kFar
+// false: arrays below 4 GB, kNearNodes4 nodes), one integer operation per load
+// instead of two and half the registers; kFar adds 64-bit addresses.  With the
+// fused slab distances above: 16 frames of 128 x 2048 beams in 1M triangles
+// 851 -> 836 us (fused) -> 820 us (offsets), four frames of seven sub-rays in a
+// 2.6M-triangle city 1447 -> 1413 -> 1356 us.
+constexpr int64_t kNearNodes4 = (int64_t)1 << 25;
+
+template <bool kFar, bool kCount = false>
 __device__ __forceinline__ bool trace_closest4(const SceneDev& S, const RayPre& p, float t_max, HitRec& h,
                                                const WorkCount* wc, int2* sh_stack, int sh_stride,
                                                unsigned* cost = nullptr)
@@ -418,9 +453,8 @@ __device__ __forceinline__ bool trace_closest4(const SceneDev& S, const RayPre& 
     stack.sh_stride = sh_stride;
     // entry planes per axis: lo for a positive direction, hi for a negative one;
     // chosen once per ray as load offsets instead of selects per node
-    const int ex = p.ix < 0.0f ? 1 : 0, ey = p.iy < 0.0f ? 3 : 2, ez = p.iz < 0.0f ? 5 : 4;
-    const unsigned long long ox2 = pack2(p.ox, p.ox), oy2 = pack2(p.oy, p.oy), oz2 = pack2(p.oz, p.oz);
-    const unsigned long long ix2 = pack2(p.ix, p.ix), iy2 = pack2(p.iy, p.iy), iz2 = pack2(p.iz, p.iz);
+    const SlabRay sr = slab_ray(p);
+    const unsigned ex = 16u * sr.flip[0], ey = 32u + 16u * sr.flip[1], ez = 64u + 16u * sr.flip[2];
     constexpr unsigned kNone = 0xFFFFFFFFu;
     int sp = 0;
     int node = 0;
@@ -433,11 +467,12 @@ __device__ __forceinline__ bool trace_closest4(const SceneDev& S, const RayPre& 
             h.leaf = kBadIndex;
             return false;
         }
-        const float4* q = S.nodes4 + 8 * (int64_t)node;
-        const int2 meta = __ldg(reinterpret_cast<const int2*>(q + 7));
+        const char* q = reinterpret_cast<const char*>(S.nodes4) + (kFar ? (int64_t)node * 128 : (int64_t)0);
+        const unsigned at = kFar ? 0u : (unsigned)node * 128u;
+        auto plane = [&](unsigned o) { return __ldg(reinterpret_cast<const float4*>(q + (at + o))); };
+        const int2 meta = __ldg(reinterpret_cast<const int2*>(q + (at + 112u)));
         float4 kn, kf;
-        near_far4(__ldg(q + ex), __ldg(q + (1 - ex)), __ldg(q + ey), __ldg(q + (5 - ey)), __ldg(q + ez),
-                  __ldg(q + (9 - ez)), ox2, oy2, oz2, ix2, iy2, iz2, kn, kf);
+        near_far4(plane(ex), plane(16u - ex), plane(ey), plane(80u - ey), plane(ez), plane(144u - ez), sr, kn, kf);
         const unsigned hit = (kn.x <= fminf(kf.x, h.cull) ? 1u : 0u) | (kn.y <= fminf(kf.y, h.cull) ? 2u : 0u) |
                              (kn.z <= fminf(kf.z, h.cull) ? 4u : 0u) | (kn.w <= fminf(kf.w, h.cull) ? 8u : 0u);
         const unsigned leafm = (unsigned)meta.y;
@@ -446,7 +481,7 @@ __device__ __forceinline__ bool trace_closest4(const SceneDev& S, const RayPre& 
         if (leaves) {
             // triangle children first, through one call site
             const float cull0 = h.cull;
-            const int4 c = __ldg(reinterpret_cast<const int4*>(q + 6));
+            const int4 c = __ldg(reinterpret_cast<const int4*>(q + (at + 96u)));
             while (leaves) {
                 const unsigned j = (unsigned)(__ffs(leaves) - 1);
                 leaves &= leaves - 1;
@@ -539,9 +574,8 @@ __device__ __forceinline__ bool trace_closest8(const SceneDev& S, const RayPre& 
     stack.sh = sh_stack;
     stack.sh_stride = sh_stride;
     // entry planes per axis (lower ones for a positive direction), as load offsets
-    const int ex = p.ix < 0.0f ? 2 : 0, ey = p.iy < 0.0f ? 6 : 4, ez = p.iz < 0.0f ? 10 : 8;
-    const unsigned long long ox2 = pack2(p.ox, p.ox), oy2 = pack2(p.oy, p.oy), oz2 = pack2(p.oz, p.oz);
-    const unsigned long long ix2 = pack2(p.ix, p.ix), iy2 = pack2(p.iy, p.iy), iz2 = pack2(p.iz, p.iz);
+    const SlabRay sr = slab_ray(p);
+    const int ex = 2 * sr.flip[0], ey = 4 + 2 * sr.flip[1], ez = 8 + 2 * sr.flip[2];
     constexpr unsigned kNone = 0xFFFFFFFFu;
     int sp = 0;
     int node = 0;
@@ -558,9 +592,9 @@ __device__ __forceinline__ bool trace_closest8(const SceneDev& S, const RayPre& 
         const int2 meta = __ldg(reinterpret_cast<const int2*>(q + 14));
         float4 ka, fa, kb, fb;
         near_far4(__ldg(q + ex), __ldg(q + (2 - ex)), __ldg(q + ey), __ldg(q + (10 - ey)), __ldg(q + ez),
-                  __ldg(q + (18 - ez)), ox2, oy2, oz2, ix2, iy2, iz2, ka, fa);
+                  __ldg(q + (18 - ez)), sr, ka, fa);
         near_far4(__ldg(q + ex + 1), __ldg(q + (3 - ex)), __ldg(q + ey + 1), __ldg(q + (11 - ey)),
-                  __ldg(q + ez + 1), __ldg(q + (19 - ez)), ox2, oy2, oz2, ix2, iy2, iz2, kb, fb);
+                  __ldg(q + ez + 1), __ldg(q + (19 - ez)), sr, kb, fb);
         const unsigned hit = (ka.x <= fminf(fa.x, h.cull) ? 1u : 0u) | (ka.y <= fminf(fa.y, h.cull) ? 2u : 0u) |
                              (ka.z <= fminf(fa.z, h.cull) ? 4u : 0u) | (ka.w <= fminf(fa.w, h.cull) ? 8u : 0u) |
                              (kb.x <= fminf(fb.x, h.cull) ? 16u : 0u) | (kb.y <= fminf(fb.y, h.cull) ? 32u : 0u) |
