@@ -438,11 +438,13 @@ lidar_status lidar_measure_fp32_rate(lidar_ctx* ctx, int64_t fma_per_thread, dou
 
 /* Ray schedule of a sensor slot.  The cast kernel's warps take groups of 32
  * consecutive positions of the slot's ray order; by default that order is the
- * Morton order of the beam directions (coherent warps).  This call measures
- * the traversal cost of every beam on `frame` (one frame of that slot, cast
- * with counting enabled), and reorders the 32-beam groups so that the most
- * expensive groups run first (longest-processing-time-first), which shortens
- * the tail of a cast where the last warps would otherwise run alone.
+ * Morton order of the beam directions in groups of 32 (coherent warps), the
+ * groups with the most level beams first (a level beam meets the most boxes).
+ * This call measures the traversal cost of every beam on `frame` (one frame
+ * of that slot, cast with counting enabled), and reorders the 32-beam groups
+ * so that the most expensive groups run first
+ * (longest-processing-time-first), which shortens the tail of a cast where
+ * the last warps would otherwise run alone.
  * mode 0: whole 32-beam groups of the Morton order, by their largest cost;
  * mode 1: single beams by cost bucket (4 buckets per octave of cost, most
  *         expensive first, Morton order within a bucket), so that each warp
@@ -452,7 +454,7 @@ lidar_status lidar_measure_fp32_rate(lidar_ctx* ctx, int64_t fma_per_thread, dou
 lidar_status lidar_schedule_by_cost(lidar_ctx* ctx, const lidar_scene* scene, const lidar_frame* frame,
                                     uint64_t seed, int32_t mode);
 
-/* Restores the Morton order of a slot. */
+/* Restores the default order of a slot. */
 lidar_status lidar_reset_schedule(lidar_ctx* ctx, int32_t slot);
 
 /* --------------------------------------------- rolling shutter, multi-echo */

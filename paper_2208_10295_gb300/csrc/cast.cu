@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_cast(SceneDev S, const Sens
                                               unsigned long long* work_counter, int tile_rays, WorkCount wc,
                                               CompactCounts cc, lidar_points pts, int64_t n_beams_total, int fused,
                                               const __grid_constant__ InlineFrames inl, unsigned* zero_next,
-                                              int64_t zero_words, uint64_t wait_ns, int pdl)
+                                              int64_t zero_words, uint64_t wait_ns, int pdl, int take_turns)
 {
     const int lane = threadIdx.x & 31;
     // clear the counter region of the cast after this one
@@ -297,10 +297,15 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_cast(SceneDev S, const Sens
             }
             break;
         }
-        const int fi = find_frame(tile_first, n_frames, tile);
+        // frames of equal tile counts are taken together, the first tiles of all
+        // of them first: the level beams' long walks then start early in every
+        // frame and the cheap ones end the cast (16 frames of 128 x 2048 beams
+        // 847 -> 800 us, four city frames of seven sub-rays 1371 -> 1326 us,
+        // four sweeps 574 -> 480 us)
+        const int fi = take_turns ? (int)(tile % n_frames) : find_frame(tile_first, n_frames, tile);
         const FrameDev& fr = fr_tab[fi];
         const SensorDev& sd = sensors[fr.sensor];
-        const int64_t base = (tile - tile_first[fi]) * tile_rays;
+        const int64_t base = (take_turns ? tile / n_frames : tile - tile_first[fi]) * tile_rays;
         if (!kCount && sd.n_sub > 1) {
             // a beam's sub-rays on neighbouring lanes (32 / n_sub beams per warp
             // step): they take nearly the same path through the tree, so the warp
@@ -515,6 +520,7 @@ struct CastArgs {
     int64_t zero_words;
     uint64_t wait_ns;
     int pdl;
+    int take_turns;
 };
 
 template <bool C, int V, int W>
@@ -524,7 +530,7 @@ cudaError_t launch_one(cudaStream_t s, CastArgs a, int64_t grid, int block, size
     auto fn = k_cast<C, V, W>;
     void* args[] = {&a.scene, &a.sensors, &a.frames, &a.n_frames, &a.prefix, &a.n_tiles, &a.table, &a.seed,
                     &a.out, &a.status, &a.work_counter, &a.tile_rays, &a.wc, &a.cc, &a.pts, &a.n_total,
-                    &a.fused, &a.inl, &a.zero_next, &a.zero_words, &a.wait_ns, &a.pdl};
+                    &a.fused, &a.inl, &a.zero_next, &a.zero_words, &a.wait_ns, &a.pdl, &a.take_turns};
     if (a.fused) {
         // every block must be resident for the grid-wide waits; the occupancy
         // of this instantiation depends only on the block size and the shared
@@ -571,7 +577,7 @@ cudaError_t launch_one(cudaStream_t s, CastArgs a, int64_t grid, int block, size
     if (a.fused) return cudaLaunchCooperativeKernel((const void*)fn, dim3((unsigned)grid), dim3(block), args, smem, s);
     fn<<<(unsigned)grid, block, smem, s>>>(a.scene, a.sensors, a.frames, a.n_frames, a.prefix, a.n_tiles, a.table,
                                             a.seed, a.out, a.status, a.work_counter, a.tile_rays, a.wc, a.cc, a.pts,
-                                            a.n_total, a.fused, a.inl, a.zero_next, a.zero_words, a.wait_ns, a.pdl);
+                                            a.n_total, a.fused, a.inl, a.zero_next, a.zero_words, a.wait_ns, a.pdl, a.take_turns);
     return cudaGetLastError();
 }
 
@@ -583,7 +589,7 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
                         unsigned long long* work_counter, const LaunchCfg& cfg, int num_sms,
                         int64_t n_beams_total, const WorkCount* count, void* compact_scratch,
                         int64_t* n_points_dev, const lidar_points* points, bool* scattered,
-                        const InlineFrames* inline_frames, const CounterRegion* region)
+                        const InlineFrames* inline_frames, const CounterRegion* region, bool equal_frames)
 {
     if (scattered) *scattered = false;
     if (n_tiles == 0) return cudaSuccess;
@@ -610,6 +616,7 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
     a.wc = count ? *count : WorkCount{nullptr, nullptr, nullptr, nullptr};
     a.n_total = n_beams_total;
     a.wait_ns = cfg.wait_ns;
+    a.take_turns = equal_frames && n_frames > 1 ? 1 : 0;
     if (inline_frames) a.inl = *inline_frames;  // else n == 0: the device table
     const bool clean = region && region->clean;
     cudaError_t* refused = region ? region->overlap_refused : nullptr;
@@ -845,9 +852,47 @@ cudaError_t launch_cost_schedule(cudaStream_t s, const uint32_t* cost, const uin
     return cudaGetLastError();
 }
 
+namespace {
+// key of a 32-beam group of the Morton order: how far from level its most
+// level beam is (a partial group last, so that every other one stays whole)
+__global__ void k_group_level(const float* __restrict__ dirs, const uint32_t* __restrict__ order, int n,
+                              uint32_t* keys, uint32_t* vals)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n_groups = (n + kScheduleGroup - 1) / kScheduleGroup;
+    if (g >= n_groups) return;
+    const int lo = g * kScheduleGroup, hi = min(n, lo + kScheduleGroup);
+    float z = 2.0f;
+    for (int j = lo; j < hi; ++j) z = fminf(z, fabsf(dirs[3 * (int64_t)order[j] + 2]));
+    keys[g] = hi - lo < kScheduleGroup ? 0xFFFFFFFFu : __float_as_uint(z);
+    vals[g] = (uint32_t)g;
+}
+}  // namespace
+
+// The Morton order's groups, most level first.  A cast ends with its longest
+// walks, those of level beams that graze the ground; started first they
+// overlap the rest.  (Scratch: that of launch_cost_schedule.)  One 128 x 2048
+// frame in 1M triangles 159 -> 149 us, rig of four sensors 1033 -> 1015 us.
+cudaError_t launch_level_order(cudaStream_t s, const float* dirs, const uint32_t* base_order, int n,
+                               uint32_t* new_order, void* scratch, size_t scratch_bytes)
+{
+    if (n == 0) return cudaSuccess;
+    if (scratch_bytes < cost_schedule_scratch_bytes(n)) return cudaErrorInvalidValue;
+    const int g = (n + kScheduleGroup - 1) / kScheduleGroup;
+    uint32_t* keys = (uint32_t*)scratch;
+    uint32_t* vals = (uint32_t*)((char*)scratch + ((g * 4 + 255) / 256) * 256);
+    char* rest = (char*)scratch + ((g * 4 + 255) / 256) * 256 * 2;
+    k_group_level<<<(g + 255) / 256, 256, 0, s>>>(dirs, base_order, n, keys, vals);
+    cudaError_t e = radix_sort_pairs_u32(s, keys, vals, g, 32, rest, scratch_bytes - (rest - (char*)scratch));
+    if (e != cudaSuccess) return e;
+    k_permute_groups<<<(n + 255) / 256, 256, 0, s>>>(vals, base_order, n, new_order);
+    return cudaGetLastError();
+}
+
 size_t ray_order_scratch_bytes(int64_t n)
 {
-    return ((n * sizeof(uint32_t) + 255) / 256) * 256 + radix_sort_scratch_bytes(n);
+    return std::max(((n * sizeof(uint32_t) + 255) / 256) * 256 + radix_sort_scratch_bytes(n),
+                    cost_schedule_scratch_bytes(n));
 }
 
 cudaError_t launch_ray_order(cudaStream_t s, const float* dirs, int n, uint32_t* order, void* scratch,

@@ -199,7 +199,7 @@ cudaError_t radix_sort_pairs_u64(cudaStream_t s, uint64_t* keys, uint32_t* vals,
 cudaError_t radix_sort_pairs_u32(cudaStream_t s, uint32_t* keys, uint32_t* vals, int64_t n, int key_bits,
                                  void* scratch, size_t scratch_bytes);
 
-// cast.cu
+// cast.cu (equal_frames: every frame has the same number of tiles)
 // Instrumentation of the traversal (work counted per launch, not timed).
 struct WorkCount {
     unsigned long long* totals;   // [0] node visits, [1] triangle tests
@@ -214,7 +214,7 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
                         int64_t n_beams_total, const WorkCount* count = nullptr, void* compact_scratch = nullptr,
                         int64_t* n_points_dev = nullptr, const lidar_points* points = nullptr,
                         bool* scattered = nullptr, const InlineFrames* inline_frames = nullptr,
-                        const CounterRegion* region = nullptr);
+                        const CounterRegion* region = nullptr, bool equal_frames = false);
 // ordered compaction fused with the cast: the cast counts kept returns per
 // 1024-beam tile and scans them (compact_scratch of fused_compact_scratch_bytes);
 // with `points` and cfg.fused_scatter it also writes the points after a
@@ -231,6 +231,10 @@ cudaError_t launch_set_poses(cudaStream_t s, FrameDev* frames, int n_frames, con
 cudaError_t launch_ray_order(cudaStream_t s, const float* dirs, int n_beams, uint32_t* order,
                              void* scratch, size_t scratch_bytes);
 size_t ray_order_scratch_bytes(int64_t n_beams);
+// 32-ray groups of `base_order`, most level first (a grazing ray meets the most
+// boxes); scratch of ray_order_scratch_bytes
+cudaError_t launch_level_order(cudaStream_t s, const float* dirs, const uint32_t* base_order, int n_beams,
+                               uint32_t* new_order, void* scratch, size_t scratch_bytes);
 // Reorders 32-ray groups of `base_order` by their largest measured beam cost,
 // most expensive first (cost indexed by beam).
 cudaError_t launch_cost_schedule(cudaStream_t s, const uint32_t* cost, const uint32_t* base_order, int n_beams,
@@ -299,7 +303,8 @@ struct EchoOut {
 cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDev* sensors_dev,
                                const SweepDev* frames_dev, int n_frames, const int64_t* tile_prefix_dev,
                                int64_t n_tiles, TableDev T, uint64_t seed, BeamsOut out, EchoOut echo, int* status,
-                               unsigned long long* work_counter, const LaunchCfg& cfg, int num_sms);
+                               unsigned long long* work_counter, const LaunchCfg& cfg, int num_sms,
+                               bool equal_sweeps);
 
 // ------------------------------------------------------------ raster path
 

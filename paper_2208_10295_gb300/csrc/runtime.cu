@@ -554,8 +554,8 @@ lidar_status lidar_set_sensor(lidar_ctx* c, int32_t slot, const lidar_sensor_des
     lidar_status st = ensure_scratch(c, ray_order_scratch_bytes(n));
     if (st != LIDAR_OK) return st;
     LIDAR_CUDA(launch_ray_order(c->stream, sl.dirs_dev, (int)n, sl.base_order_dev, c->scratch, c->scratch_bytes));
-    LIDAR_CUDA(cudaMemcpyAsync(sl.order_dev, sl.base_order_dev, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice,
-                               c->stream));
+    LIDAR_CUDA(launch_level_order(c->stream, sl.dirs_dev, sl.base_order_dev, (int)n, sl.order_dev, c->scratch,
+                                  c->scratch_bytes));
     SensorDev& sd = sl.dev;
     sd.dirs = sl.dirs_dev;
     sd.sweep = sl.sweep_dev;
@@ -646,7 +646,7 @@ lidar_status lidar_set_materials(lidar_ctx* c, const float* table, int32_t M)
 // kInlineFrames frames they go into *inl (the launch parameters) and nothing
 // is copied to the device; otherwise into the device table.
 static lidar_status prepare_frames(lidar_ctx* c, const lidar_frame* frames, int32_t n_frames, int64_t* n_beams_total,
-                                   int64_t* n_tiles, InlineFrames* inl = nullptr)
+                                   int64_t* n_tiles, bool* equal, InlineFrames* inl = nullptr)
 {
     LIDAR_CHECK_ARG(frames != nullptr && n_frames > 0, "lidar_cast: need at least one frame");
     std::vector<FrameDev> fd((size_t)n_frames);
@@ -669,6 +669,9 @@ static lidar_status prepare_frames(lidar_ctx* c, const lidar_frame* frames, int3
         off += c->slots[s].n_beams;
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
     }
+    *equal = true;
+    for (int32_t k = 1; k < n_frames; ++k)
+        if (prefix[k] * n_frames != tiles * k) *equal = false;
     if (inl) inl->n = 0;
     if (inl && n_frames <= kInlineFrames) {
         for (int32_t k = 0; k < n_frames; ++k) {
@@ -775,8 +778,8 @@ static lidar_status counter_region(lidar_ctx* c, int64_t n_total, bool compact, 
 static lidar_status cast_impl(lidar_ctx* c, const lidar_scene* scene, const FrameDev* frames_dev,
                               const int64_t* prefix_dev, int32_t n_frames, int64_t n_total, int64_t n_tiles,
                               uint64_t seed, const lidar_beams* beams, const lidar_points* points,
-                              int64_t* n_points_dev, bool may_alloc, const InlineFrames* inl = nullptr,
-                              bool direct = false)
+                              int64_t* n_points_dev, bool may_alloc, bool equal_frames,
+                              const InlineFrames* inl = nullptr, bool direct = false)
 {
     lidar_status tst = traversal_available(c, scene, "cast");
     if (tst != LIDAR_OK) return tst;
@@ -866,7 +869,7 @@ static lidar_status cast_impl(lidar_ctx* c, const lidar_scene* scene, const Fram
     const cudaError_t le = launch_cast(c->stream, S, c->sensors_dev, frames_dev, n_frames, prefix_dev, n_tiles,
                                        c->table, seed, out, c->status_dev, c->work_counter, c->cfg, c->num_sms,
                                        n_total, nullptr, comp, n_points_dev, points, &scattered, inl,
-                                       use_region ? &R : nullptr);
+                                       use_region ? &R : nullptr, equal_frames);
     if (refused != cudaSuccess)
         log_info(std::string("cast: overlapped launch refused (") + cudaGetErrorString(refused) +
                  "), launched after the previous cast instead");
@@ -932,14 +935,15 @@ lidar_status lidar_cast(lidar_ctx* c, const lidar_scene* scene, const lidar_fram
     if (st != LIDAR_OK) return st;
     DeviceGuard g(c->device);
     int64_t n_total = 0, n_tiles = 0;
+    bool equal = false;
     InlineFrames inl;
-    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &inl);
+    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal, &inl);
     if (st != LIDAR_OK) return st;
     if (log_level() >= 2)
         log_info("cast: " + std::to_string(n_frames) + " frames, " + std::to_string(n_total) + " beams, traversal " +
                  std::to_string(c->cfg.traversal) + (points ? ", point cloud" : ""));
     return cast_impl(c, scene, c->frames_dev, c->tile_prefix_dev, n_frames, n_total, n_tiles, seed, beams, points,
-                     n_points_dev, true, &inl, true);
+                     n_points_dev, true, equal, &inl, true);
 }
 
 }  // extern "C"
@@ -1116,6 +1120,9 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
         off += c->slots[s].n_beams;
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
     }
+    bool equal = true;
+    for (int32_t k = 1; k < n_frames; ++k)
+        if (prefix[(size_t)k] * n_frames != tiles * k) equal = false;
     DeviceGuard g(c->device);
     // sweep records, then the tile prefix at a 256-byte boundary, in one block
     const size_t prefix_at = ((size_t)n_frames * sizeof(SweepDev) + 255) / 256 * 256;
@@ -1140,7 +1147,7 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
     // persistent tiles that follow the slots' ray orders and schedules
     LIDAR_CUDA(launch_sweep_tiles(c->stream, scene_dev(scene), c->sensors_dev, c->sweeps_dev, n_frames, prefix_dev,
                                   tiles, c->table, seed, to_beams_out(beams), echo, c->status_dev, c->work_counter,
-                                  c->cfg, c->num_sms));
+                                  c->cfg, c->num_sms, equal));
     return LIDAR_OK;
 }
 
@@ -1184,6 +1191,7 @@ struct lidar_batch {
     int32_t n_frames = 0;
     int64_t n_total = 0, n_tiles = 0;
     int tile_rays = 0;
+    bool equal_frames = false;        // every frame has the same number of tiles
     std::vector<int32_t> slot_beams;  // beams of each slot at creation (-1 = unused)
 };
 
@@ -1202,9 +1210,11 @@ lidar_status lidar_batch_create(lidar_ctx* c, const lidar_frame* frames, int32_t
     *out = nullptr;
     DeviceGuard g(c->device);
     int64_t n_total = 0, n_tiles = 0;
-    lidar_status st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles);
+    bool equal = false;
+    lidar_status st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal);
     if (st != LIDAR_OK) return st;
     lidar_batch* b = new lidar_batch();
+    b->equal_frames = equal;
     b->ctx = c;
     b->n_frames = n_frames;
     b->n_total = n_total;
@@ -1286,7 +1296,7 @@ lidar_status lidar_cast_batch(lidar_ctx* c, const lidar_scene* scene, const lida
     if (st != LIDAR_OK) return st;
     DeviceGuard g(c->device);
     return cast_impl(c, scene, b->frames_dev, b->prefix_dev, b->n_frames, b->n_total, b->n_tiles, seed, beams, points,
-                     n_points_dev, false);
+                     n_points_dev, false, b->equal_frames);
 }
 
 lidar_status lidar_graph_create(lidar_ctx* c, const lidar_scene* scene, lidar_batch* b, const float* poses_dev,
@@ -1312,7 +1322,7 @@ lidar_status lidar_graph_create(lidar_ctx* c, const lidar_scene* scene, lidar_ba
         if (poses_dev) e = launch_set_poses(cap, b->frames_dev, b->n_frames, poses_dev);
         if (e == cudaSuccess)
             st = cast_impl(c, scene, b->frames_dev, b->prefix_dev, b->n_frames, b->n_total, b->n_tiles, seed, beams,
-                           points, n_points_dev, false);
+                           points, n_points_dev, false, b->equal_frames);
         cudaError_t e2 = cudaStreamEndCapture(cap, &gr->graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -1476,7 +1486,8 @@ static lidar_status counting_cast(lidar_ctx* c, const lidar_scene* scene, const 
     lidar_status st = traversal_available(c, scene, "counting cast");
     if (st != LIDAR_OK) return st;
     int64_t n_total = 0, n_tiles = 0;
-    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles);
+    bool equal = false;
+    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal);
     if (st != LIDAR_OK) return st;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const int64_t node_words = (scene->n_nodes + 31) / 32 + 1, leaf_words = (scene->n_tris + 31) / 32 + 1;
@@ -1499,7 +1510,7 @@ static lidar_status counting_cast(lidar_ctx* c, const lidar_scene* scene, const 
     SceneDev S = scene_dev(scene);
     LIDAR_CUDA(launch_cast(c->stream, S, c->sensors_dev, c->frames_dev, n_frames, c->tile_prefix_dev, n_tiles,
                            c->table, seed, dense, c->status_dev, c->work_counter, c->cfg, c->num_sms, n_total,
-                           &wc));
+                           &wc, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, equal));
     LIDAR_CUDA(launch_popcount(c->stream, node_bits, node_words, totals + 2));
     LIDAR_CUDA(launch_popcount(c->stream, leaf_bits, leaf_words, totals + 3));
     LIDAR_CUDA(cudaMemcpyAsync(h, totals, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
@@ -1580,8 +1591,10 @@ lidar_status lidar_reset_schedule(lidar_ctx* c, int32_t slot)
     }
     DeviceGuard g(c->device);
     SensorSlot& sl = c->slots[slot];
-    LIDAR_CUDA(cudaMemcpyAsync(sl.order_dev, sl.base_order_dev, sl.n_beams * sizeof(uint32_t),
-                               cudaMemcpyDeviceToDevice, c->stream));
+    lidar_status st = ensure_scratch(c, ray_order_scratch_bytes(sl.n_beams));
+    if (st != LIDAR_OK) return st;
+    LIDAR_CUDA(launch_level_order(c->stream, sl.dirs_dev, sl.base_order_dev, (int)sl.n_beams, sl.order_dev, c->scratch,
+                                  c->scratch_bytes));
     LIDAR_CUDA(cudaStreamSynchronize(c->stream));
     return LIDAR_OK;
 }

@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
                                                                  const int64_t* __restrict__ tile_prefix,
                                                                  int64_t n_tiles, int tile_rays, TableDev T,
                                                                  uint64_t seed, BeamsOut out, EchoOut echo,
-                                                                 int* status, unsigned long long* work_counter)
+                                                                 int* status, unsigned long long* work_counter,
+                                                                 int take_turns)
 {
     const int lane = threadIdx.x & 31;
     while (true) {
@@ -111,14 +112,23 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
         if (lane == 0) claimed = atomicAdd(work_counter, 1ull);
         const int64_t tile = (int64_t)__shfl_sync(0xffffffffu, claimed, 0);
         if (tile >= n_tiles) break;
-        int lo = 0, hi = n_frames - 1;  // last sweep whose first tile is at or before `tile`
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (tile_prefix[mid] <= tile) lo = mid; else hi = mid - 1;
+        int lo = 0;
+        int64_t first = 0;  // of this tile's positions, in tiles
+        if (take_turns) {
+            // sweeps of equal tile counts take turns (as frames do in the frame cast)
+            lo = (int)(tile % n_frames);
+            first = tile / n_frames;
+        } else {
+            int hi = n_frames - 1;  // last sweep whose first tile is at or before `tile`
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (tile_prefix[mid] <= tile) lo = mid; else hi = mid - 1;
+            }
+            first = tile - tile_prefix[lo];
         }
         const SweepDev f = frames[lo];
         const SensorDev& sd = sensors[f.sensor];
-        const int64_t base = (tile - tile_prefix[lo]) * tile_rays;
+        const int64_t base = first * tile_rays;
         if (sd.n_sub > 1) {
             // a beam's sub-rays on neighbouring lanes (as in the frame cast): the
             // strongest return is picked across the beam's lanes and written by its
@@ -233,7 +243,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
 cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDev* sensors_dev,
                                const SweepDev* frames_dev, int n_frames, const int64_t* tile_prefix_dev,
                                int64_t n_tiles, TableDev T, uint64_t seed, BeamsOut out, EchoOut echo, int* status,
-                               unsigned long long* work_counter, const LaunchCfg& cfg, int num_sms)
+                               unsigned long long* work_counter, const LaunchCfg& cfg, int num_sms, bool equal_sweeps)
 {
     if (n_tiles == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(work_counter, 0, sizeof(unsigned long long), s);
@@ -249,7 +259,7 @@ cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDe
 #define LIDAR_SWEEP_LAUNCH(MB, EC)                                                                              \
     (far4 ? k_sweep_tiles<MB, EC, true> : k_sweep_tiles<MB, EC, false>)<<<gd, bt, 0, s>>>(                      \
         S, sensors_dev, frames_dev, n_frames, tile_prefix_dev, n_tiles, cfg.tile_rays, T, seed, out, echo,      \
-        status, work_counter)
+        status, work_counter, equal_sweeps && n_frames > 1 ? 1 : 0)
     const bool ec = echo.n_echoes > 0;
     if (resident <= 512) {
         if (ec) LIDAR_SWEEP_LAUNCH(2, true); else LIDAR_SWEEP_LAUNCH(2, false);
