@@ -529,9 +529,10 @@ typedef struct {
 /* Dense per-beam outputs like lidar_cast (beams required; points are not
  * produced): tri = the triangle seen through the beam's pixel centre, t = the
  * range before noise, normal = 0 (the G-buffer has no normal), mat = the
- * 8-bit stencil, inst = the 24-bit colour, sub = 0.  Frames are rendered one
- * after another in the context's scratch (about 16 + 4 bytes per pixel per
- * camera plus 3 bytes per triangle and camera).  Asynchronous. */
+ * 8-bit stencil, inst = the 24-bit colour, sub = 0.  Only pixels that a beam
+ * reads are rendered.  Frames are rendered one after another in the context's
+ * scratch (about 8 bytes per pixel per camera plus 3 bytes per triangle and
+ * camera).  Asynchronous. */
 lidar_status lidar_raster_cast(lidar_ctx* ctx, const lidar_scene* scene, const lidar_frame* frames_host,
                                int32_t n_frames, uint64_t seed, const lidar_raster_config* cfg,
                                const lidar_beams* beams);

@@ -337,14 +337,19 @@ struct GBuffer {
 };
 
 size_t raster_big_capacity(int n_cameras, int64_t n_tris);
-size_t raster_scratch_bytes(int width, int n_cameras, int64_t n_tris, bool with_tri);
+// what is rasterised: the pixels that beams read, or whole images (with the
+// triangles seen)
+enum RasterUse { RASTER_BEAMS, RASTER_IMAGES, RASTER_IMAGES_TRI };
+size_t raster_scratch_bytes(int width, int n_cameras, int64_t n_tris, RasterUse use);
 cudaError_t launch_invert_leaf_order(cudaStream_t s, const uint32_t* leaf_tri, int64_t n, uint32_t* orig_to_leaf);
 // rasterises one frame's K images into scratch (raster_scratch_bytes); *G
 // receives the G-buffer's location inside it (with_tri: also the triangles)
 cudaError_t launch_rasterise(cudaStream_t s, const SceneDev& S, const RasterCams& C, const RasterFrame& F,
                              const uint32_t* orig_to_leaf, void* scratch, bool with_tri, GBuffer* G, int num_sms);
-cudaError_t launch_resample(cudaStream_t s, const RasterCams& C, const RasterFrame& F, const SensorDev* sensors_dev,
-                            int sensor, int n_beams, int frame_id, int64_t beam_offset, TableDev T, uint64_t seed,
-                            const GBuffer& G, BeamsOut out);
+// one frame of a sensor: rasterises the pixels its beams read, and reads them
+cudaError_t launch_raster_beams(cudaStream_t s, const SceneDev& S, const RasterCams& C, const RasterFrame& F,
+                                const uint32_t* orig_to_leaf, void* scratch, const SensorDev* sensors_dev, int sensor,
+                                int n_beams, int frame_id, int64_t beam_offset, TableDev T, uint64_t seed,
+                                BeamsOut out, int num_sms);
 
 }  // namespace lidar

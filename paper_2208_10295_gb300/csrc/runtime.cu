@@ -951,7 +951,7 @@ lidar_status lidar_cast(lidar_ctx* c, const lidar_scene* scene, const lidar_fram
 // ------------------------------------------------------------ raster path
 
 static lidar_status raster_setup(lidar_ctx* c, const lidar_scene* scene, const lidar_raster_config* cfg,
-                                 bool with_tri, RasterCams& C)
+                                 RasterUse use, RasterCams& C)
 {
     LIDAR_CHECK_ARG(c != nullptr && scene != nullptr && cfg != nullptr, "raster: NULL argument");
     LIDAR_CHECK_ARG(scene->ctx == c, "raster: scene belongs to another context");
@@ -978,7 +978,7 @@ static lidar_status raster_setup(lidar_ctx* c, const lidar_scene* scene, const l
         }
         LIDAR_CUDA(launch_invert_leaf_order(c->stream, sc->leaf_tri, sc->n_tris, sc->orig_to_leaf));
     }
-    return ensure_scratch(c, raster_scratch_bytes(C.W, C.K, scene->n_tris, with_tri));
+    return ensure_scratch(c, raster_scratch_bytes(C.W, C.K, scene->n_tris, use));
 }
 
 static RasterFrame raster_frame(const RasterCams& C, const lidar_frame& fr, float t_max)
@@ -1023,18 +1023,16 @@ lidar_status lidar_raster_cast(lidar_ctx* c, const lidar_scene* scene, const lid
     DeviceGuard g(c->device);
     RasterCams C;
     const BeamsOut out = to_beams_out(beams);
-    st = raster_setup(c, scene, cfg, out.tri != nullptr, C);
+    st = raster_setup(c, scene, cfg, RASTER_BEAMS, C);
     if (st != LIDAR_OK) return st;
     const SceneDev S = scene_dev(scene);
     int64_t offset = 0;
     for (int32_t k = 0; k < n_frames; ++k) {
         const SensorSlot& sl = c->slots[frames[k].sensor];
         const RasterFrame F = raster_frame(C, frames[k], sl.dev.t_max);
-        GBuffer G{};
-        LIDAR_CUDA(launch_rasterise(c->stream, S, C, F, scene->orig_to_leaf, c->scratch, out.tri != nullptr, &G,
-                                    c->num_sms));
-        LIDAR_CUDA(launch_resample(c->stream, C, F, c->sensors_dev, frames[k].sensor, (int)sl.n_beams, frames[k].frame,
-                                   offset, c->table, seed, G, out));
+        LIDAR_CUDA(launch_raster_beams(c->stream, S, C, F, scene->orig_to_leaf, c->scratch, c->sensors_dev,
+                                       frames[k].sensor, (int)sl.n_beams, frames[k].frame, offset, c->table, seed, out,
+                                       c->num_sms));
         offset += sl.n_beams;
     }
     return LIDAR_OK;
@@ -1167,7 +1165,7 @@ lidar_status lidar_raster_gbuffer(lidar_ctx* c, const lidar_scene* scene, const 
         LIDAR_CHECK_ARG(isfinite(frame->pose[j]), "lidar_raster_gbuffer: non-finite pose");
     DeviceGuard g(c->device);
     RasterCams C;
-    lidar_status st = raster_setup(c, scene, cfg, tri_dev != nullptr, C);
+    lidar_status st = raster_setup(c, scene, cfg, tri_dev != nullptr ? RASTER_IMAGES_TRI : RASTER_IMAGES, C);
     if (st != LIDAR_OK) return st;
     const RasterFrame F = raster_frame(C, *frame, c->slots[s].dev.t_max);
     GBuffer G{};
