@@ -34,6 +34,17 @@ def _frames_array(frames):
     return fr
 
 
+def _as_signed(a, signed):
+    """Host integers as the signed type of the same width torch holds them in;
+    arrays of that width are reinterpreted, not copied."""
+    a = np.asarray(a)
+    signed = np.dtype(signed)
+    if a.dtype.kind in "iu" and a.dtype.itemsize == signed.itemsize and a.dtype.isnative and a.flags.c_contiguous \
+            and a.flags.writeable:
+        return a.view(signed)
+    return a.astype(signed)
+
+
 class Scene:
     def __init__(self, lidar, handle, n_tris):
         self._lidar = lidar
@@ -95,11 +106,11 @@ class Lidar:
     # ----------------------------------------------------------- scene
     def build_scene(self, verts, tris, mat=None, inst=None) -> Scene:
         verts = torch.as_tensor(verts, dtype=torch.float32, device=self.device).contiguous()
-        tris = torch.as_tensor(np.asarray(tris).astype(np.int32) if isinstance(tris, np.ndarray) else tris,
+        tris = torch.as_tensor(_as_signed(tris, np.int32) if isinstance(tris, np.ndarray) else tris,
                                device=self.device).to(torch.int32).contiguous()
         n = tris.shape[0]
-        mat_t = None if mat is None else torch.as_tensor(np.asarray(mat).astype(np.int16), device=self.device)
-        inst_t = None if inst is None else torch.as_tensor(np.asarray(inst).astype(np.int32), device=self.device)
+        mat_t = None if mat is None else torch.as_tensor(_as_signed(mat, np.int16), device=self.device)
+        inst_t = None if inst is None else torch.as_tensor(_as_signed(inst, np.int32), device=self.device)
         h = ctypes.c_void_p()
         C.check(C.lidar_scene_build(self.handle, _ptr(verts), verts.shape[0], _ptr(tris), n, _ptr(mat_t),
                                     _ptr(inst_t), ctypes.byref(h)), "lidar_scene_build")
