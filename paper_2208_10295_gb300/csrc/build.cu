@@ -1012,12 +1012,15 @@ struct CollapseDP {
     AreaW w;                  // face weights of the area measure (also the largest-area rule's)
 };
 
-__global__ void k_parents(const float4* __restrict__ bn, int n_binary, int* parent_node, int* parent_leaf)
+// (and, with `internal`, how many of each node's children are internal)
+__global__ void k_parents(const float4* __restrict__ bn, int n_binary, int* parent_node, int* parent_leaf,
+                          unsigned* internal)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= n_binary) return;
     const float4 n3 = bn[4 * (int64_t)n + 3];
     const int c[2] = {__float_as_int(n3.x), __float_as_int(n3.y)};
+    if (internal) internal[n] = (c[0] >= 0 ? 1u : 0u) + (c[1] >= 0 ? 1u : 0u);
     for (int k = 0; k < 2; ++k) {
         // (a build that failed may have left any bits here)
         if (c[k] >= 0 && c[k] < n_binary) parent_node[c[k]] = n;
@@ -1390,7 +1393,7 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
         const int nb = (int)n_binary;
         e = cudaMemsetAsync(c.parent_node, 0xFF, (size_t)nb * sizeof(int), s);
         if (e != cudaSuccess) return e;
-        k_parents<<<(nb + 255) / 256, 256, 0, s>>>(binary_nodes, nb, c.parent_node, c.parent_leaf);
+        k_parents<<<(nb + 255) / 256, 256, 0, s>>>(binary_nodes, nb, c.parent_node, c.parent_leaf, nullptr);
         for (int k = 0; k < 2; ++k) {
             const CollapseDP& dp = c.a.tree[k].dp;
             e = cudaMemsetAsync(dp.visits, 0, (size_t)nb * sizeof(unsigned), s);
@@ -1467,14 +1470,18 @@ struct TreeletArgs {
     int n_leaves;
     int n_binary;
     float4* nodes;            // binary nodes, rewritten in place
-    const int* parent_node;   // [n_binary], -1 at the root
-    const int* parent_leaf;   // [n_leaves]
-    unsigned* visits;         // [n_binary] children finished, zero at the start of a round
+    int* parent;              // [n_binary], -1 at the root; kept up to date by the rewrites
+    // A round visits the nodes below which something may change: all of them in
+    // round 1, then those that the round before rewrote and their ancestors.
+    uint8_t* on_path;         // [n_binary] the last round (from 2) that visits the node
+    unsigned* expect;         // [n_binary] children the round visits
+    unsigned* visits;         // [n_binary] of these, finished; zero at the start of a round
     float* cost;              // [n_binary] surface-area cost of each node's subtree
-    // A treelet is a function of its subtree alone, so one that was kept and
-    // whose subtree is as it was is kept again without a look: mark[n] is the
-    // last round (1, 2, ...) that rewrote node n, up[n] the last one that
-    // rewrote a treelet of n's subtree before n was reached.
+    // A treelet is a function of its subtree alone (the costs of its leaves
+    // among it, to the last bit), so one that was kept and whose subtree is as
+    // it was is kept again without a look: mark[n] is the last round (1, 2,
+    // ...) that rewrote node n, up[n] the last one that changed a node or a
+    // cost of n's subtree before it was done with n.
     uint8_t* mark;            // [n_binary]
     uint8_t* up;              // [n_binary]
     int round;
@@ -1609,7 +1616,8 @@ __device__ __forceinline__ void merge_partition(float& best, int& bq, int width)
 // treelet's leaf i while it grows; the areas of its 127 subsets are spread over
 // the lanes, four each; the dynamic program runs size by size, one subset per
 // lane up to five leaves, four lanes a subset at six, all lanes on the whole.
-// 1: rewritten, 0: kept, -1: a child reference out of range.
+// 1: rewritten, or its cost changed; 0: all as it was; -1: a child reference out
+// of range.
 //
 // A leaf that is an internal node has its own record in flight as soon as it
 // joins the treelet, so that opening it later waits for no load.
@@ -1687,10 +1695,6 @@ __device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, in
     }
     // the node's cost in its current shape
     const float c_now = a.c_node * root_area + __shfl_sync(kAll, first_cost, 0) + __shfl_sync(kAll, first_cost, 1);
-    if (k < 3) {
-        if (lane == 0) a.cost[node] = c_now;
-        return 0;
-    }
     __syncwarp();  // the treelet before this one is done with the shared arrays
     if (lane < k) {
         for (int j = 0; j < 3; ++j) {
@@ -1787,8 +1791,12 @@ __device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, in
     // one of the shapes the program compares, so it is never dearer beyond
     // rounding)
     if (!(t.c[full] < c_now * (1.0f - 1e-5f))) {
-        if (lane == 0) a.cost[node] = c_now;
-        return 0;
+        bool moved = false;
+        if (lane == 0) {
+            moved = __float_as_int(__ldcg(&a.cost[node])) != __float_as_int(c_now);
+            a.cost[node] = c_now;
+        }
+        return __any_sync(kAll, moved) ? 1 : 0;
     }
     // rewrite: subset S at internal node id, its parts as leaves or the next
     // internal nodes of the treelet (one lane lays out the shape, then a lane
@@ -1831,6 +1839,8 @@ __device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, in
             make_float4(__int_as_float(t.out_ref[0][lane]), __int_as_float(t.out_ref[1][lane]), 0.0f, 0.0f);
         a.cost[id] = t.c[s];
         a.mark[id] = (uint8_t)a.round;
+        for (int side = 0; side < 2; ++side)
+            if (t.out_ref[side][lane] >= 0) a.parent[t.out_ref[side][lane]] = id;
     }
     return 1;
 }
@@ -1843,24 +1853,54 @@ __device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, in
 constexpr int kTreeletThreads = 32;
 constexpr int kTreeletBlocks = 16;
 
-// A lane per triangle climbs; the lanes that are second at their node have
-// the warp process those nodes' treelets one after another.
+// The nodes the round rewrote and all above them: the nodes the next one
+// visits, and how many of each one's children are among them.
+__global__ void __launch_bounds__(kBuildThreads) k_treelet_paths(TreeletArgs a)
+{
+    int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= a.n_binary || a.mark[n] != a.round - 1) return;
+    for (int step = 0; n >= 0 && step < kTreeletMaxClimb; ++step) {
+        // bytes have no atomics: the word that holds the node's
+        unsigned* word = (unsigned*)(a.on_path + (n & ~3));
+        const unsigned shift = 8u * (n & 3);
+        unsigned seen = *(volatile unsigned*)word;
+        while (((seen >> shift) & 0xFFu) != (unsigned)a.round) {
+            const unsigned want = (seen & ~(0xFFu << shift)) | ((unsigned)a.round << shift);
+            const unsigned was = atomicCAS(word, seen, want);
+            if (was == seen) break;
+            seen = was;
+        }
+        if (((seen >> shift) & 0xFFu) == (unsigned)a.round) return;  // the rest of the path is taken
+        n = a.parent[n];
+        if (n >= a.n_binary) {
+            raise_status(a.status, ST_BOUNDS);
+            return;
+        }
+        if (n >= 0) atomicAdd(&a.expect[n], 1u);
+    }
+}
+
+// A lane per node: those none of whose children the round visits climb from
+// there, each going on from a node when it is the last of the visited children
+// to finish; the lanes whose node needs a look have the warp process the
+// treelets one after another.
 //
 // What bounds it: the chain of each warp's treelets (issue ~40 %, ~1,000 warp
-// instructions and ~7,000 cycles a treelet) in the first round, and in later
-// ones, which look at few treelets, the climb itself (an arrival, a fence and
-// two loads a level).  Measured at 0.65M triangles (city, eight rounds): one
-// thread a treelet with its program in local memory 9.4 ms a round; by a warp
-// 1.2 ms; with the treelets whose subtree is unchanged kept unseen 1.2, 0.88,
-// 0.64, 0.51, 0.41, 0.35, 0.31, 0.30 ms.
+// instructions and ~7,000 cycles a treelet) in the first round, the climb (an
+// arrival, a fence and two loads a level) in later ones, which look at few
+// treelets.  Measured at 0.65M triangles (city, eight rounds): one thread a
+// treelet with its program in local memory 9.4 ms a round; by a warp 1.2 ms;
+// with the treelets whose subtree is unchanged kept unseen 1.2, 0.88, 0.64,
+// 0.51, 0.41, 0.35, 0.31, 0.30 ms; climbing only where something was rewritten
+// 1.2, 0.85, 0.62, 0.43, 0.35, 0.30, 0.24, 0.25 ms.
 __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_round(TreeletArgs a)
 {
     __shared__ TreeletShared s_t[kTreeletThreads / 32];
     TreeletShared& t = s_t[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int sub2 = lane < 21 ? kSubsets2[lane] : 0, sub3a = kSubsets3[lane], sub3b = lane < 3 ? kSubsets3[32 + lane] : 0;
-    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    int node = leaf < a.n_leaves ? a.parent_leaf[leaf] : -1;
+    int node = blockIdx.x * blockDim.x + threadIdx.x;
+    if (node >= a.n_binary || (a.round > 1 && a.on_path[node] != a.round) || a.expect[node] != 0u) node = -1;
     for (int step = 0;; ++step) {
         if (node >= a.n_binary || (node >= 0 && step >= kTreeletMaxClimb)) {
             raise_status(a.status, ST_BOUNDS);
@@ -1872,11 +1912,12 @@ __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_rou
         int parent = -1;
         bool look = false, below = false;  // the warp has to look at the treelet; its subtree changed this round
         if (node >= 0) {
-            const unsigned before = atomicAdd(&a.visits[node], 1u);
+            const unsigned before = step > 0 ? atomicAdd(&a.visits[node], 1u) + 1u : 0u;
+            const unsigned expect = a.expect[node];
             c = __ldcg(reinterpret_cast<const int2*>(&a.nodes[4 * (int64_t)node + 3]));
-            parent = a.parent_node[node];
+            parent = __ldcg(&a.parent[node]);
             look = a.round == 1 || __ldcg(&a.mark[node]) == a.round - 1;
-            if (before == 0u) node = -1;  // the other child is still running
+            if (before != expect) node = -1;  // another child is still running
         }
         if (!__any_sync(0xffffffffu, node >= 0)) return;
         climb_fence();  // the children's results are visible to the warp
@@ -1895,19 +1936,22 @@ __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_rou
                 treelet_child(a.nodes, node, 1, ref, R);
                 const float cost = subtree_cost(a, c.x, L), other = subtree_cost(a, c.y, R);
                 tbox_grow(L, R);
-                a.cost[node] = a.c_node * tbox_area(L, a.w) + cost + other;
+                const float now = a.c_node * tbox_area(L, a.w) + cost + other;
+                below = __float_as_int(__ldcg(&a.cost[node])) != __float_as_int(now);
+                a.cost[node] = now;
                 look = false;
             }
         } else {
             below = (c.x >= 0 && __ldcg(&a.up[c.x]) == a.round) || (c.y >= 0 && __ldcg(&a.up[c.y]) == a.round);
             look = look || below;
+            below = false;
         }
         for (unsigned todo = __ballot_sync(0xffffffffu, look); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
             const int did = treelet_node(a, __shfl_sync(0xffffffffu, node, src), t, sub2, sub3a, sub3b);
             if (lane == src) {
                 if (did < 0) raise_status(a.status, ST_BOUNDS);
-                below = below || did > 0;
+                below = did > 0;
             }
         }
         if (below) a.up[node] = (uint8_t)a.round;
@@ -1946,8 +1990,8 @@ __global__ void k_parents_reset(int* parent_node, int n_binary)
 
 size_t treelet_scratch_bytes(int64_t n_tris)
 {
-    // parents of nodes and leaves, visit counters, costs, marks
-    return 4 * align256(n_tris * sizeof(int)) + 2 * align256(n_tris);
+    // parents of nodes and leaves, expected and finished children, costs, path, mark and up bytes
+    return 5 * align256(n_tris * sizeof(int)) + 3 * align256(n_tris);
 }
 
 cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, float4* nodes, int* max_height_dev,
@@ -1962,27 +2006,33 @@ cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, 
     char* p = (char*)scratch;
     int* parent_node = (int*)p; p += align256(n * sizeof(int));
     int* parent_leaf = (int*)p; p += align256(n * sizeof(int));
+    unsigned* expect = (unsigned*)p; p += align256(n * sizeof(int));
     unsigned* visits = (unsigned*)p; p += align256(n * sizeof(int));
     float* cost = (float*)p; p += align256(n * sizeof(float));
+    uint8_t* on_path = (uint8_t*)p; p += align256(n);
     uint8_t* mark = (uint8_t*)p; p += align256(n);
-    uint8_t* up = (uint8_t*)p;
+    uint8_t* up = (uint8_t*)p; p += align256(n);
     const int nb_blocks = (n_binary + 255) / 256;
-    TreeletArgs a{tris, (int)n, n_binary, nodes, parent_node, parent_leaf, visits, cost, mark, up, 0, treelets_dev, status,
-                  1.0f, tri_cost, area_w};
-    e = cudaMemsetAsync(mark, 0, (size_t)((char*)up + n - (char*)mark), s);
+    TreeletArgs a{tris, (int)n, n_binary, nodes, parent_node, on_path, expect, visits, cost, mark, up, 0, treelets_dev,
+                  status, 1.0f, tri_cost, area_w};
+    e = cudaMemsetAsync(on_path, 0, (size_t)(p - (char*)on_path), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(expect, 0, (size_t)((char*)cost - (char*)expect), s);
     if (e != cudaSuccess) return e;
+    k_parents_reset<<<nb_blocks, 256, 0, s>>>(parent_node, n_binary);
+    k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf, expect);
     for (int r = 0; r < rounds; ++r) {
         a.round = r + 1;
-        k_parents_reset<<<nb_blocks, 256, 0, s>>>(parent_node, n_binary);
-        k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf);
-        e = cudaMemsetAsync(visits, 0, (size_t)n_binary * sizeof(unsigned), s);
-        if (e != cudaSuccess) return e;
-        k_treelet_round<<<(int)((n + kTreeletThreads - 1) / kTreeletThreads), kTreeletThreads, 0, s>>>(a);
+        if (r > 0) {
+            e = cudaMemsetAsync(expect, 0, (size_t)((char*)cost - (char*)expect), s);  // and visits
+            if (e != cudaSuccess) return e;
+            k_treelet_paths<<<nb_blocks, kBuildThreads, 0, s>>>(a);
+        }
+        k_treelet_round<<<(n_binary + kTreeletThreads - 1) / kTreeletThreads, kTreeletThreads, 0, s>>>(a);
     }
     // parents and root height of the final shape (every box a rewrite stored is
     // the exact union of the boxes below it)
     k_parents_reset<<<nb_blocks, 256, 0, s>>>(parent_node, n_binary);
-    k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf);
+    k_parents<<<nb_blocks, 256, 0, s>>>(nodes, n_binary, parent_node, parent_leaf, nullptr);
     e = cudaMemsetAsync(max_height_dev, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     k_root_height<<<(int)((n + kBuildThreads - 1) / kBuildThreads), kBuildThreads, 0, s>>>(
