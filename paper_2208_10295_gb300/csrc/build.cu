@@ -1239,7 +1239,9 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
 }
 
 // Even blocks walk the 4-wide tree, odd ones the 8-wide: the levels of the two
-// hide each other's waits.  Measured at 1M triangles, both trees: see collapse_plan.
+// hide each other's waits.  Bound by those: 1M triangles, both trees, 17 and 11
+// levels, 2.6 ms with three launches and a host round trip a level and one
+// block scanning it, 0.28 ms so.
 __global__ void __launch_bounds__(kCollapseThreads) k_collapse_levels(const __grid_constant__ CollapseArgs a)
 {
     // a build that failed left no tree to walk
@@ -1405,7 +1407,11 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
         if (e != cudaSuccess) return e;
     }
     // two blocks (one a tree, which meet nobody) for what one block's tiles hold
-    const int64_t want = 2 * ((n_binary / 4 + kCollapseThreads - 1) / kCollapseThreads);
+    // and one a tree and SM at most: a level's two meetings cost more with more
+    // blocks than its widest tiles gain (1M triangles: 1,646 us for a rebuild and
+    // cast, 1,661 with two, 1,702 with three)
+    const int64_t want = std::min<int64_t>(2 * ((n_binary / 4 + kCollapseThreads - 1) / kCollapseThreads),
+                                           2 * (int64_t)num_sms);
     const int grid =
         std::max(2, coop_blocks((const void*)k_collapse_levels, kCollapseThreads, 0, num_sms, coop, want) / 2 * 2);
     if (grid == 2) {
