@@ -131,13 +131,20 @@ __device__ __forceinline__ void intersect_triangle(const float4* __restrict__ tr
     const float A0 = __fsub_rn(a.x, p.ox), A1 = __fsub_rn(a.y, p.oy), A2 = __fsub_rn(a.z, p.oz);
     const float B0 = __fsub_rn(b.x, p.ox), B1 = __fsub_rn(b.y, p.oy), B2 = __fsub_rn(b.z, p.oz);
     const float C0 = __fsub_rn(c.x, p.ox), C1 = __fsub_rn(c.y, p.oy), C2 = __fsub_rn(c.z, p.oz);
-    const float Akz = sel3(A0, A1, A2, p.kz), Bkz = sel3(B0, B1, B2, p.kz), Ckz = sel3(C0, C1, C2, p.kz);
-    const float Ax = __fmaf_rn(-p.Sx, Akz, sel3(A1, A2, A0, p.kz));
-    const float Ay = __fmaf_rn(-p.Sy, Akz, sel3(A2, A0, A1, p.kz));
-    const float Bx = __fmaf_rn(-p.Sx, Bkz, sel3(B1, B2, B0, p.kz));
-    const float By = __fmaf_rn(-p.Sy, Bkz, sel3(B2, B0, B1, p.kz));
-    const float Cx = __fmaf_rn(-p.Sx, Ckz, sel3(C1, C2, C0, p.kz));
-    const float Cy = __fmaf_rn(-p.Sy, Ckz, sel3(C2, C0, C1, p.kz));
+    // a branch a warp mostly takes one way, for two selects per coordinate
+    float Ax, Ay, Akz, Bx, By, Bkz, Cx, Cy, Ckz;
+    auto shear = [&](float x, float y, float z, float& X, float& Y, float& Z) {
+        Z = z;
+        X = __fmaf_rn(-p.Sx, z, x);
+        Y = __fmaf_rn(-p.Sy, z, y);
+    };
+    if (p.kz == 0) {
+        shear(A1, A2, A0, Ax, Ay, Akz); shear(B1, B2, B0, Bx, By, Bkz); shear(C1, C2, C0, Cx, Cy, Ckz);
+    } else if (p.kz == 1) {
+        shear(A2, A0, A1, Ax, Ay, Akz); shear(B2, B0, B1, Bx, By, Bkz); shear(C2, C0, C1, Cx, Cy, Ckz);
+    } else {
+        shear(A0, A1, A2, Ax, Ay, Akz); shear(B0, B1, B2, Bx, By, Bkz); shear(C0, C1, C2, Cx, Cy, Ckz);
+    }
     // edge functions, antisymmetric under swapping the edge's end points
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
