@@ -560,6 +560,10 @@ typedef struct {
                                 wait (cooperative launch); 0: as a separate kernel */
 } lidar_launch_config;
 
+/* The default is 128 threads x 4 blocks.  Until a call sets block_threads or
+ * blocks_per_sm to another value, casts and sweeps with traversal 2 choose how
+ * many threads to keep resident by the number of rays (512 a SM for few, up to
+ * 1,024 for many); afterwards they run as set, the default values included. */
 lidar_status lidar_get_launch_config(lidar_ctx* ctx, lidar_launch_config* out);
 lidar_status lidar_set_launch_config(lidar_ctx* ctx, const lidar_launch_config* cfg);
 

@@ -146,6 +146,7 @@ struct lidar_ctx {
     int dense_cur = 0;       // which half of the scratch the next direct cast's dense records use
     std::vector<std::pair<uintptr_t, uintptr_t>> last_out;  // output byte ranges of the last direct cast
     LaunchCfg cfg{128, 4, 32, 1, 2, 1};
+    bool own_shape = true;    // nobody has set another block_threads or blocks_per_sm: see launch_shape
     int build_method = 1;     // 0 Karras LBVH, 1 PLOC clustering (fewer node fetches per ray)
     int ploc_radius = 16;
     int collapse = 0;         // wide nodes: 0 open the largest child, 1 SAH dynamic program
@@ -690,12 +691,39 @@ lidar_status lidar_set_materials(lidar_ctx* c, const float* table, int32_t M)
     return LIDAR_OK;
 }
 
+// Launch configuration of a cast or sweep of `ray_tiles` (32 rays each).  As
+// long as no caller has set block_threads or blocks_per_sm to anything but the
+// default, the library chooses how many threads stay resident: few tiles end
+// with their longest walks, which want the fewest neighbours (512 threads a
+// SM); many are bound by issue and want the most warps (1,024 at 64
+// registers).  Measured with the 4-wide walk, us, 512 / 768 / 1,024 threads a
+// SM: 8,192 tiles (a 128 x 2048 frame in 1M triangles) 108 / 107 / 116, 16,384
+// 158 / 152 / 158, 32,768 286 / 251 / 253, 65,536 571 / 484 / 453; a city's
+// 57,344 (seven sub-rays) 421 / 386 / 426, 114,688 773 / 682 / 667; a rig's
+// 31,000 294 / 269 / 267, 123,000 1024 / 876 / 833.  256-thread blocks took 1-8
+// % less than 128-thread ones at each.
+static LaunchCfg launch_shape(const lidar_ctx* c, int64_t ray_tiles)
+{
+    LaunchCfg cfg = c->cfg;
+    if (!c->own_shape || cfg.traversal != 2) return cfg;
+    const int64_t warps = (int64_t)c->num_sms * 16;  // resident at 512 threads a SM
+    cfg.block_threads = 256;
+    cfg.blocks_per_sm = ray_tiles < 8 * warps ? 2 : (ray_tiles < 32 * warps ? 3 : 4);
+    return cfg;
+}
+
+// What the frames of a cast have in common
+struct FrameMix {
+    bool equal = false;      // every frame has the same number of tiles
+    int64_t ray_tiles = 0;   // 32-ray tiles in all, sub-rays counted
+};
+
 // shared front half of the cast entry points
 // Frame records and tile prefix of a cast.  With `inl` and at most
 // kInlineFrames frames they go into *inl (the launch parameters) and nothing
 // is copied to the device; otherwise into the device table.
 static lidar_status prepare_frames(lidar_ctx* c, const lidar_frame* frames, int32_t n_frames, int64_t* n_beams_total,
-                                   int64_t* n_tiles, bool* equal, InlineFrames* inl = nullptr)
+                                   int64_t* n_tiles, FrameMix* mix, InlineFrames* inl = nullptr)
 {
     LIDAR_CHECK_ARG(frames != nullptr && n_frames > 0, "lidar_cast: need at least one frame");
     std::vector<FrameDev> fd((size_t)n_frames);
@@ -717,10 +745,11 @@ static lidar_status prepare_frames(lidar_ctx* c, const lidar_frame* frames, int3
         prefix[k] = tiles;
         off += c->slots[s].n_beams;
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
+        mix->ray_tiles += (c->slots[s].n_beams + 31) / 32 * c->slots[s].dev.n_sub;
     }
-    *equal = true;
+    mix->equal = true;
     for (int32_t k = 1; k < n_frames; ++k)
-        if (prefix[k] * n_frames != tiles * k) *equal = false;
+        if (prefix[k] * n_frames != tiles * k) mix->equal = false;
     if (inl) inl->n = 0;
     if (inl && n_frames <= kInlineFrames) {
         for (int32_t k = 0; k < n_frames; ++k) {
@@ -827,7 +856,7 @@ static lidar_status counter_region(lidar_ctx* c, int64_t n_total, bool compact, 
 static lidar_status cast_impl(lidar_ctx* c, const lidar_scene* scene, const FrameDev* frames_dev,
                               const int64_t* prefix_dev, int32_t n_frames, int64_t n_total, int64_t n_tiles,
                               uint64_t seed, const lidar_beams* beams, const lidar_points* points,
-                              int64_t* n_points_dev, bool may_alloc, bool equal_frames,
+                              int64_t* n_points_dev, bool may_alloc, const FrameMix& mix,
                               const InlineFrames* inl = nullptr, bool direct = false)
 {
     lidar_status tst = traversal_available(c, scene, "cast");
@@ -916,9 +945,9 @@ static lidar_status cast_impl(lidar_ctx* c, const lidar_scene* scene, const Fram
     cudaError_t refused = cudaSuccess;
     R.overlap_refused = &refused;
     const cudaError_t le = launch_cast(c->stream, S, c->sensors_dev, frames_dev, n_frames, prefix_dev, n_tiles,
-                                       c->table, seed, out, c->status_dev, c->work_counter, c->cfg, c->num_sms,
-                                       n_total, nullptr, comp, n_points_dev, points, &scattered, inl,
-                                       use_region ? &R : nullptr, equal_frames);
+                                       c->table, seed, out, c->status_dev, c->work_counter,
+                                       launch_shape(c, mix.ray_tiles), c->num_sms, n_total, nullptr, comp, n_points_dev, points, &scattered, inl,
+                                       use_region ? &R : nullptr, mix.equal);
     if (refused != cudaSuccess)
         log_info(std::string("cast: overlapped launch refused (") + cudaGetErrorString(refused) +
                  "), launched after the previous cast instead");
@@ -984,15 +1013,15 @@ lidar_status lidar_cast(lidar_ctx* c, const lidar_scene* scene, const lidar_fram
     if (st != LIDAR_OK) return st;
     DeviceGuard g(c->device);
     int64_t n_total = 0, n_tiles = 0;
-    bool equal = false;
+    FrameMix mix;
     InlineFrames inl;
-    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal, &inl);
+    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &mix, &inl);
     if (st != LIDAR_OK) return st;
     if (log_level() >= 2)
         log_info("cast: " + std::to_string(n_frames) + " frames, " + std::to_string(n_total) + " beams, traversal " +
                  std::to_string(c->cfg.traversal) + (points ? ", point cloud" : ""));
     return cast_impl(c, scene, c->frames_dev, c->tile_prefix_dev, n_frames, n_total, n_tiles, seed, beams, points,
-                     n_points_dev, true, equal, &inl, true);
+                     n_points_dev, true, mix, &inl, true);
 }
 
 }  // extern "C"
@@ -1168,8 +1197,12 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
     }
     bool equal = true;
-    for (int32_t k = 1; k < n_frames; ++k)
+    int64_t ray_tiles = 0;
+    for (int32_t k = 0; k < n_frames; ++k) {
         if (prefix[(size_t)k] * n_frames != tiles * k) equal = false;
+        const SensorSlot& sl = c->slots[frames[k].sensor];
+        ray_tiles += (sl.n_beams + 31) / 32 * sl.dev.n_sub;
+    }
     DeviceGuard g(c->device);
     // sweep records, then the tile prefix at a 256-byte boundary, in one block
     const size_t prefix_at = ((size_t)n_frames * sizeof(SweepDev) + 255) / 256 * 256;
@@ -1194,7 +1227,7 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
     // persistent tiles that follow the slots' ray orders and schedules
     LIDAR_CUDA(launch_sweep_tiles(c->stream, scene_dev(scene), c->sensors_dev, c->sweeps_dev, n_frames, prefix_dev,
                                   tiles, c->table, seed, to_beams_out(beams), echo, c->status_dev, c->work_counter,
-                                  c->cfg, c->num_sms, equal));
+                                  launch_shape(c, ray_tiles), c->num_sms, equal));
     return LIDAR_OK;
 }
 
@@ -1238,7 +1271,7 @@ struct lidar_batch {
     int32_t n_frames = 0;
     int64_t n_total = 0, n_tiles = 0;
     int tile_rays = 0;
-    bool equal_frames = false;        // every frame has the same number of tiles
+    FrameMix mix;
     std::vector<int32_t> slot_beams;  // beams of each slot at creation (-1 = unused)
 };
 
@@ -1257,11 +1290,11 @@ lidar_status lidar_batch_create(lidar_ctx* c, const lidar_frame* frames, int32_t
     *out = nullptr;
     DeviceGuard g(c->device);
     int64_t n_total = 0, n_tiles = 0;
-    bool equal = false;
-    lidar_status st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal);
+    FrameMix mix;
+    lidar_status st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &mix);
     if (st != LIDAR_OK) return st;
     lidar_batch* b = new lidar_batch();
-    b->equal_frames = equal;
+    b->mix = mix;
     b->ctx = c;
     b->n_frames = n_frames;
     b->n_total = n_total;
@@ -1343,7 +1376,7 @@ lidar_status lidar_cast_batch(lidar_ctx* c, const lidar_scene* scene, const lida
     if (st != LIDAR_OK) return st;
     DeviceGuard g(c->device);
     return cast_impl(c, scene, b->frames_dev, b->prefix_dev, b->n_frames, b->n_total, b->n_tiles, seed, beams, points,
-                     n_points_dev, false, b->equal_frames);
+                     n_points_dev, false, b->mix);
 }
 
 lidar_status lidar_graph_create(lidar_ctx* c, const lidar_scene* scene, lidar_batch* b, const float* poses_dev,
@@ -1369,7 +1402,7 @@ lidar_status lidar_graph_create(lidar_ctx* c, const lidar_scene* scene, lidar_ba
         if (poses_dev) e = launch_set_poses(cap, b->frames_dev, b->n_frames, poses_dev);
         if (e == cudaSuccess)
             st = cast_impl(c, scene, b->frames_dev, b->prefix_dev, b->n_frames, b->n_total, b->n_tiles, seed, beams,
-                           points, n_points_dev, false, b->equal_frames);
+                           points, n_points_dev, false, b->mix);
         cudaError_t e2 = cudaStreamEndCapture(cap, &gr->graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -1533,8 +1566,8 @@ static lidar_status counting_cast(lidar_ctx* c, const lidar_scene* scene, const 
     lidar_status st = traversal_available(c, scene, "counting cast");
     if (st != LIDAR_OK) return st;
     int64_t n_total = 0, n_tiles = 0;
-    bool equal = false;
-    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &equal);
+    FrameMix mix;
+    st = prepare_frames(c, frames, n_frames, &n_total, &n_tiles, &mix);
     if (st != LIDAR_OK) return st;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const int64_t node_words = (scene->n_nodes + 31) / 32 + 1, leaf_words = (scene->n_tris + 31) / 32 + 1;
@@ -1557,7 +1590,7 @@ static lidar_status counting_cast(lidar_ctx* c, const lidar_scene* scene, const 
     SceneDev S = scene_dev(scene);
     LIDAR_CUDA(launch_cast(c->stream, S, c->sensors_dev, c->frames_dev, n_frames, c->tile_prefix_dev, n_tiles,
                            c->table, seed, dense, c->status_dev, c->work_counter, c->cfg, c->num_sms, n_total,
-                           &wc, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, equal));
+                           &wc, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, mix.equal));
     LIDAR_CUDA(launch_popcount(c->stream, node_bits, node_words, totals + 2));
     LIDAR_CUDA(launch_popcount(c->stream, leaf_bits, leaf_words, totals + 3));
     LIDAR_CUDA(cudaMemcpyAsync(h, totals, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
@@ -1706,6 +1739,7 @@ lidar_status lidar_set_launch_config(lidar_ctx* c, const lidar_launch_config* cf
     LIDAR_CHECK_ARG(cfg->fused_scatter == 0 || cfg->fused_scatter == 1,
                     "lidar_set_launch_config: fused_scatter is 0 or 1");
     DeviceGuard g(c->device);
+    if (cfg->block_threads != c->cfg.block_threads || cfg->blocks_per_sm != c->cfg.blocks_per_sm) c->own_shape = false;
     c->cfg.block_threads = cfg->block_threads;
     c->cfg.blocks_per_sm = cfg->blocks_per_sm;
     c->cfg.tile_rays = cfg->tile_rays;
