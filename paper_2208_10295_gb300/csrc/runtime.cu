@@ -154,7 +154,8 @@ struct lidar_ctx {
     int treelet_rounds = 0;   // rounds of treelet restructuring of the binary tree
     AreaW area_w{1.0f, 1.0f, 1.0f};  // face weights of the builders' area measure
     std::set<lidar_scene*> scenes;
-    cudaMemPool_t pool = nullptr;  // the scenes' arrays (NULL: cudaMalloc)
+    cudaMemPool_t pool = nullptr;  // the scenes' arrays, made with the first scene (NULL: cudaMalloc)
+    bool pool_tried = false;
 };
 
 namespace {
@@ -216,6 +217,10 @@ cudaMemPool_t create_pool(int device)
 
 cudaError_t scene_alloc(lidar_ctx* c, void** p, size_t bytes)
 {
+    if (!c->pool_tried) {
+        c->pool = create_pool(c->device);
+        c->pool_tried = true;
+    }
     if (!c->pool) return dev_alloc(p, bytes);
     *p = nullptr;
     if (alloc_fault()) return cudaErrorMemoryAllocation;
@@ -298,11 +303,9 @@ lidar_status lidar_create(int device, void* cuda_stream, lidar_ctx** out)
     static_assert(sizeof(BuildResult) <= 64, "fits between the work counter and the adjoint's");
     c->adj_arrivals = (unsigned long long*)((char*)p + 192);
     c->coop = coop;
-    c->pool = create_pool(device);
     e = dev_alloc((void**)&c->sensors_dev, sizeof(SensorDev) * LIDAR_MAX_SENSORS);
     if (e != cudaSuccess) {
         cudaFree(p);
-        if (c->pool) cudaMemPoolDestroy(c->pool);
         delete c;
         set_error("lidar_create: device allocation failed");
         return LIDAR_ENOMEM;
@@ -313,7 +316,6 @@ lidar_status lidar_create(int device, void* cuda_stream, lidar_ctx** out)
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
         cudaFree(p);
         cudaFree(c->sensors_dev);
-        if (c->pool) cudaMemPoolDestroy(c->pool);
         delete c;
         set_error("lidar_create: stream synchronisation failed");
         return LIDAR_ECUDA;
