@@ -108,6 +108,23 @@ __device__ __forceinline__ RayPre prepare_ray(const RayW& r)
     return p;
 }
 
+// Three-input FP32 max / min (sm_100+): the same result as the two-input
+// fmaxf / fminf chains, NaN inputs ignored unless all are NaN, in one
+// instruction and one dependent step instead of two.
+__device__ __forceinline__ float max3f(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+__device__ __forceinline__ float min3f(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 struct HitRec {
     float t;
     float cull;       // t * kBestScale: boxes entering beyond this are pruned
@@ -149,13 +166,13 @@ __device__ __forceinline__ void intersect_triangle(const float4* __restrict__ tr
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if (U == 0.0f || V == 0.0f || W == 0.0f) {
+    if (min3f(fabsf(U), fabsf(V), fabsf(W)) == 0.0f) {
         // exact products in double decide edge cases consistently
         U = (float)((double)Cx * (double)By - (double)Cy * (double)Bx);
         V = (float)((double)Ax * (double)Cy - (double)Ay * (double)Cx);
         W = (float)((double)Bx * (double)Ay - (double)By * (double)Ax);
     }
-    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return;
+    if (min3f(U, V, W) < 0.0f && max3f(U, V, W) > 0.0f) return;
     const float det = __fadd_rn(__fadd_rn(U, V), W);
     if (det == 0.0f) return;
     const float Az = __fmul_rn(p.Sz, Akz), Bz = __fmul_rn(p.Sz, Bkz), Cz = __fmul_rn(p.Sz, Ckz);
@@ -377,23 +394,6 @@ __device__ __forceinline__ void slab4_planes(float4 e, float4 x, unsigned long l
     unpack2(fma2(pack2(e.z, e.w), inv, near), tin.z, tin.w);
     unpack2(fma2(pack2(x.x, x.y), inv, far), tout.x, tout.y);
     unpack2(fma2(pack2(x.z, x.w), inv, far), tout.z, tout.w);
-}
-
-// Three-input FP32 max / min (sm_100+): the same result as the two-input
-// fmaxf / fminf chains, NaN inputs ignored unless all are NaN, in one
-// instruction and one dependent step instead of two.
-__device__ __forceinline__ float max3f(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
-__device__ __forceinline__ float min3f(float a, float b, float c)
-{
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
 }
 
 // Near and far slab distances of four child boxes (entry and exit planes per
