@@ -302,10 +302,12 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_cast(SceneDev S, const Sens
         // frame and the cheap ones end the cast (16 frames of 128 x 2048 beams
         // 847 -> 800 us, four city frames of seven sub-rays 1371 -> 1326 us,
         // four sweeps 574 -> 480 us)
-        const int fi = take_turns ? (int)(tile % n_frames) : find_frame(tile_first, n_frames, tile);
+        const unsigned turn = (unsigned)tile / (unsigned)n_frames;
+        const int fi = take_turns ? (int)((unsigned)tile - turn * (unsigned)n_frames)
+                                  : find_frame(tile_first, n_frames, tile);
         const FrameDev& fr = fr_tab[fi];
         const SensorDev& sd = sensors[fr.sensor];
-        const int64_t base = (take_turns ? tile / n_frames : tile - tile_first[fi]) * tile_rays;
+        const int64_t base = (take_turns ? (int64_t)turn : tile - tile_first[fi]) * tile_rays;
         if (!kCount && sd.n_sub > 1) {
             // a beam's sub-rays on neighbouring lanes (32 / n_sub beams per warp
             // step): they take nearly the same path through the tree, so the warp
@@ -616,7 +618,7 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
     a.wc = count ? *count : WorkCount{nullptr, nullptr, nullptr, nullptr};
     a.n_total = n_beams_total;
     a.wait_ns = cfg.wait_ns;
-    a.take_turns = equal_frames && n_frames > 1 ? 1 : 0;
+    a.take_turns = equal_frames && n_frames > 1 && n_tiles < ((int64_t)1 << 32) ? 1 : 0;  // (32-bit division)
     if (inline_frames) a.inl = *inline_frames;  // else n == 0: the device table
     const bool clean = region && region->clean;
     cudaError_t* refused = region ? region->overlap_refused : nullptr;

@@ -116,8 +116,9 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_sweep_tiles(SceneDev S, con
         int64_t first = 0;  // of this tile's positions, in tiles
         if (take_turns) {
             // sweeps of equal tile counts take turns (as frames do in the frame cast)
-            lo = (int)(tile % n_frames);
-            first = tile / n_frames;
+            const unsigned turn = (unsigned)tile / (unsigned)n_frames;
+            lo = (int)((unsigned)tile - turn * (unsigned)n_frames);
+            first = (int64_t)turn;
         } else {
             int hi = n_frames - 1;  // last sweep whose first tile is at or before `tile`
             while (lo < hi) {
@@ -259,7 +260,7 @@ cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDe
 #define LIDAR_SWEEP_LAUNCH(MB, EC)                                                                              \
     (far4 ? k_sweep_tiles<MB, EC, true> : k_sweep_tiles<MB, EC, false>)<<<gd, bt, 0, s>>>(                      \
         S, sensors_dev, frames_dev, n_frames, tile_prefix_dev, n_tiles, cfg.tile_rays, T, seed, out, echo,      \
-        status, work_counter, equal_sweeps && n_frames > 1 ? 1 : 0)
+        status, work_counter, equal_sweeps && n_frames > 1 && n_tiles < ((int64_t)1 << 32) ? 1 : 0)
     const bool ec = echo.n_echoes > 0;
     if (resident <= 512) {
         if (ec) LIDAR_SWEEP_LAUNCH(2, true); else LIDAR_SWEEP_LAUNCH(2, false);
