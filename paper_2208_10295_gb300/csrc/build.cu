@@ -967,38 +967,9 @@ __device__ __forceinline__ void binary_child(const float4* __restrict__ bn, int 
 __device__ __forceinline__ float half_area(const ChildBox& c, AreaW w)
 {
     const float dx = c.hi[0] - c.lo[0], dy = c.hi[1] - c.lo[1], dz = c.hi[2] - c.lo[2];
-    return w.z * dx * dy + w.x * dy * dz + w.y * dz * dx;
-}
-
-// children of binary node b; returns the number of internal ones
-template <int W>
-__device__ int gather_children(const float4* __restrict__ bn, int b, ChildBox ch[W], int& count, AreaW w)
-{
-    float area[W];  // of the children that can be opened
-    auto take = [&](int node, int side, int k) {
-        binary_child(bn, node, side, ch[k]);
-        area[k] = ch[k].ref >= 0 ? half_area(ch[k], w) : -2.0f;
-    };
-    take(b, 0, 0);
-    take(b, 1, 1);
-    count = 2;
-    while (count < W) {
-        int best = -1;
-        float best_a = -1.0f;
-        for (int k = 0; k < count; ++k)
-            if (area[k] > best_a) {
-                best_a = area[k];
-                best = k;
-            }
-        if (best < 0) break;
-        const int open = ch[best].ref;
-        take(open, 0, best);
-        take(open, 1, count);
-        ++count;
-    }
-    int internal = 0;
-    for (int k = 0; k < count; ++k) internal += ch[k].ref >= 0;
-    return internal;
+    // rounded alike wherever it is compiled: the levels and the nodes are to
+    // choose the same children
+    return fmaf(__fmul_rn(w.y, dz), dx, fmaf(__fmul_rn(w.z, dx), dy, __fmul_rn(__fmul_rn(w.x, dy), dz)));
 }
 
 // ---- SAH-optimal choice of a wide node's children (a dynamic program over the
@@ -1101,44 +1072,120 @@ __global__ void k_collapse_dp(const float4* __restrict__ bn, int n_leaves, Colla
     }
 }
 
-// children of binary node b chosen by the dynamic program; returns the number
-// of internal ones
+// How much a child of `slots` slots wants to be opened (-2: not at all): of a
+// node's children the first of the largest is, until there are W or none can be.
 template <int W>
-__device__ int gather_children_dp(const float4* __restrict__ bn, int b, const CollapseDP& dp, ChildBox ch[W],
-                                  int& count)
+__device__ __forceinline__ float open_key(const ChildBox& c, int slots, const CollapseDP& dp, int use_dp)
 {
-    int budget[W];
-    binary_child(bn, b, 0, ch[0]);
-    binary_child(bn, b, 1, ch[1]);
-    const int j = dp.split[(int64_t)b * W + W - 1];
-    budget[0] = j;
-    budget[1] = W - j;
+    if (c.ref < 0) return -2.0f;
+    if (use_dp) return slots >= 2 && !((dp.single[c.ref] >> slots) & 1u) ? 1.0f : -2.0f;
+    const float v = half_area(c, dp.w);
+    return v > -1.0f ? v : -2.0f;
+}
+
+// slots of binary node b's left child, of the `slots` that b has
+template <int W>
+__device__ __forceinline__ int left_slots(const CollapseDP& dp, int use_dp, int b, int slots)
+{
+    return use_dp ? dp.split[(int64_t)b * W + slots - 1] : 0;
+}
+
+// References of the children of the wide node at binary node b, by one thread;
+// returns the number of internal ones.  The loops are unrolled, so that all is
+// in registers: the levels of 1M triangles took 293 us with the children's
+// boxes in local memory, 223 us so.
+template <int W>
+__device__ int gather_refs(const float4* __restrict__ bn, int b, const CollapseDP& dp, int use_dp, int ref[W], int& count)
+{
+    float key[W];
+    int slots[W];
+    ChildBox c;
+    auto take = [&](int node, int side, int budget, int& r, float& k) {
+        binary_child(bn, node, side, c);
+        r = c.ref;
+        k = open_key<W>(c, budget, dp, use_dp);
+    };
+    slots[0] = left_slots<W>(dp, use_dp, b, W);
+    slots[1] = W - slots[0];
+    take(b, 0, slots[0], ref[0], key[0]);
+    take(b, 1, slots[1], ref[1], key[1]);
     count = 2;
-    for (bool more = true; more;) {
-        more = false;
-        for (int k = 0; k < count; ++k) {
-            const int x = ch[k].ref, i = budget[k];
-            if (x < 0 || i < 2 || ((dp.single[x] >> i) & 1u)) continue;
-            const int jx = dp.split[(int64_t)x * W + i - 1];
-            binary_child(bn, x, 0, ch[k]);
-            binary_child(bn, x, 1, ch[count]);
-            budget[k] = jx;
-            budget[count] = i - jx;
-            ++count;
-            more = true;
-            break;
-        }
+#pragma unroll
+    for (int at = 2; at < W; ++at) {
+        float top = -1.0f;
+        int open = -1, budget = 0;
+#pragma unroll
+        for (int k = 0; k < at; ++k)
+            if (key[k] > top) {
+                top = key[k];
+                open = ref[k];
+                budget = slots[k];
+            }
+        if (top == -1.0f) break;
+        const int left = left_slots<W>(dp, use_dp, open, budget);
+        int r;
+        float key_left;
+        take(open, 0, left, r, key_left);
+        bool found = false;
+#pragma unroll
+        for (int k = 0; k < at; ++k)
+            if (!found && key[k] == top) {
+                found = true;
+                ref[k] = r;
+                key[k] = key_left;
+                slots[k] = left;
+            }
+        slots[at] = budget - left;
+        take(open, 1, slots[at], ref[at], key[at]);
+        count = at + 1;
     }
     int internal = 0;
-    for (int k = 0; k < count; ++k) internal += ch[k].ref >= 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) internal += k < count && ref[k] >= 0;
     return internal;
 }
 
+// This lane's child of the wide node at binary node b, by the W lanes of a
+// group (the same b in each; < 0: no node), the same ones in the same order.
+// All 32 lanes call it; returns the number of children.
 template <int W>
-__device__ __forceinline__ int gather(const float4* __restrict__ bn, int b, const CollapseDP& dp, int use_dp,
-                                      ChildBox ch[W], int& count)
+__device__ int gather_lanes(const float4* __restrict__ bn, int b, const CollapseDP& dp, int use_dp, ChildBox& c)
 {
-    return use_dp ? gather_children_dp<W>(bn, b, dp, ch, count) : gather_children<W>(bn, b, ch, count, dp.w);
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & (W - 1);
+    int count = b >= 0 ? 2 : 0, slots = 0;
+    float key = -2.0f;
+    for (int a = 0; a < 3; ++a) {
+        c.lo[a] = INFINITY;
+        c.hi[a] = -INFINITY;
+    }
+    c.ref = -1;
+    auto take = [&](int node, int side, int budget) {
+        const int left = left_slots<W>(dp, use_dp, node, budget);
+        slots = side ? budget - left : left;
+        binary_child(bn, node, side, c);
+        key = open_key<W>(c, slots, dp, use_dp);
+    };
+    if (lane < count) take(b, lane, W);
+    for (;;) {
+        float top = count < W ? key : -2.0f;
+        int best = lane;
+#pragma unroll
+        for (int d = 1; d < W; d *= 2) {
+            const float other = __shfl_xor_sync(kAll, top, d);
+            const int at = __shfl_xor_sync(kAll, best, d);
+            if (other > top || (other == top && at < best)) {
+                top = other;
+                best = at;
+            }
+        }
+        const bool more = top > -1.0f;
+        if (!__any_sync(kAll, more)) return count;
+        const int open = __shfl_sync(kAll, c.ref, best, W);
+        const int budget = __shfl_sync(kAll, slots, best, W);
+        if (more && (lane == best || lane == count)) take(open, lane != best, budget);
+        count += more;
+    }
 }
 
 constexpr int kCollapseThreads = 256;
@@ -1178,13 +1225,13 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
             const int i = t * T + tid;
             int internal = 0;
             if (i < n) {
-                ChildBox ch[W];
-                int count;
+                int ref[W], count;
                 const int slot = base + i;
-                internal = gather<W>(a.bn, slot ? __ldcg(&c.root[slot]) : 0, c.dp, a.use_dp, ch, count);
+                internal = gather_refs<W>(a.bn, slot ? __ldcg(&c.root[slot]) : 0, c.dp, a.use_dp, ref, count);
                 int m = 0;
-                for (int k = 0; k < count; ++k)
-                    if (ch[k].ref >= 0) __stcg(&c.kids[(int64_t)i * W + m++], ch[k].ref);
+#pragma unroll
+                for (int k = 0; k < W; ++k)
+                    if (k < count && ref[k] >= 0) __stcg(&c.kids[(int64_t)i * W + m++], ref[k]);
                 __stcg(&c.first[slot], internal);
                 need = max(need, (slot ? __ldcg(&c.pushes[slot]) : 0) + (internal > 0 ? internal - 1 : 0));
             }
@@ -1252,7 +1299,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
 // Even blocks walk the 4-wide tree, odd ones the 8-wide: the levels of the two
 // hide each other's waits.  Bound by those: 1M triangles, both trees, 17 and 11
 // levels, 2.6 ms with three launches and a host round trip a level and one
-// block scanning it, 0.28 ms so.
+// block scanning it, 0.22 ms so.
 __global__ void __launch_bounds__(kCollapseThreads) k_collapse_levels(const __grid_constant__ CollapseArgs a)
 {
     // a build that failed left no tree to walk
@@ -1261,7 +1308,10 @@ __global__ void __launch_bounds__(kCollapseThreads) k_collapse_levels(const __gr
     else collapse_levels<8>(a, a.tree[1], blockIdx.x >> 1, gridDim.x >> 1);
 }
 
-// every node of a wide tree, a thread each
+// Every node of a wide tree, a lane per child.  Bound by the loads of the
+// opened nodes, one after another, and by the stores: with a thread per node,
+// its children in local memory and 16-byte stores 128 or 256 bytes apart, 1M
+// triangles took 108 us (8-wide) and 74 us (4-wide); so, 46 and 38 us.
 template <int W>
 __global__ void __launch_bounds__(kCollapseThreads) k_collapse_nodes(const float4* __restrict__ bn, int n,
                                                                      const int* __restrict__ root,
@@ -1269,53 +1319,27 @@ __global__ void __launch_bounds__(kCollapseThreads) k_collapse_nodes(const float
                                                                      float4* __restrict__ nodes, const CollapseDP dp,
                                                                      int use_dp)
 {
-    constexpr int G = W / 4;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    ChildBox ch[W];
-    int count;
-    gather<W>(bn, i ? root[i] : 0, dp, use_dp, ch, count);
+    const int lane = threadIdx.x & (W - 1), group = threadIdx.x & 31 & ~(W - 1);
+    const int64_t i = ((int64_t)blockIdx.x * kCollapseThreads + threadIdx.x) / W;
+    const bool live = i < n;
+    ChildBox c;
+    const int count = gather_lanes<W>(bn, live ? (i ? root[i] : 0) : -1, dp, use_dp, c);
+    const unsigned inner = (__ballot_sync(0xffffffffu, c.ref >= 0) >> group) & ((1u << W) - 1u);
+    if (!live) return;
+    // internal children first, keeping their order (a stable partition)
+    const unsigned below = (1u << lane) - 1u;
+    const int n_inner = __popc(inner), rank = __popc(inner & below);
     const int next = first[i];
-    {
-        // internal children first, keeping their order (a stable partition)
-        ChildBox tmp[W];
-        int m = 0;
-        for (int k = 0; k < count; ++k)
-            if (ch[k].ref >= 0) tmp[m++] = ch[k];
-        for (int k = 0; k < count; ++k)
-            if (ch[k].ref < 0) tmp[m++] = ch[k];
-        for (int k = 0; k < count; ++k) ch[k] = tmp[k];
+    const int k = lane >= count ? lane : (c.ref >= 0 ? rank : n_inner + lane - rank);
+    const int code = lane >= count ? 0 : (c.ref >= 0 ? next + rank : c.ref);
+    float* out = reinterpret_cast<float*>(nodes) + 8 * W * i + k;
+    for (int a = 0; a < 3; ++a) {
+        out[2 * a * W] = c.lo[a];
+        out[(2 * a + 1) * W] = c.hi[a];
     }
-    float lo[3][W], hi[3][W];
-    int code[W];
-    int k_int = 0;
-    unsigned leaf_mask = 0;
-    for (int k = 0; k < W; ++k) {
-        if (k < count) {
-            for (int a = 0; a < 3; ++a) { lo[a][k] = ch[k].lo[a]; hi[a][k] = ch[k].hi[a]; }
-            if (ch[k].ref >= 0) {
-                code[k] = next + k_int++;
-            } else {
-                code[k] = ch[k].ref;
-                leaf_mask |= 1u << k;
-            }
-        } else {
-            for (int a = 0; a < 3; ++a) { lo[a][k] = INFINITY; hi[a][k] = -INFINITY; }
-            code[k] = 0;
-        }
-    }
-    float4* out = nodes + 8 * G * (int64_t)i;
-    for (int g = 0; g < G; ++g) {
-        const int c = 4 * g;
-        for (int a = 0; a < 3; ++a) {
-            out[(2 * a) * G + g] = make_float4(lo[a][c], lo[a][c + 1], lo[a][c + 2], lo[a][c + 3]);
-            out[(2 * a + 1) * G + g] = make_float4(hi[a][c], hi[a][c + 1], hi[a][c + 2], hi[a][c + 3]);
-        }
-        out[6 * G + g] = make_float4(__int_as_float(code[c]), __int_as_float(code[c + 1]),
-                                     __int_as_float(code[c + 2]), __int_as_float(code[c + 3]));
-        out[7 * G + g] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-    out[7 * G] = make_float4(__int_as_float(next), __int_as_float((int)leaf_mask), 0.0f, 0.0f);
+    out[6 * W] = __int_as_float(code);
+    const int leaf_mask = (int)(((1u << count) - 1u) & ~((1u << n_inner) - 1u));
+    out[7 * W] = k == 0 ? __int_as_float(next) : (k == 1 ? __int_as_float(leaf_mask) : 0.0f);
 }
 
 }  // namespace
@@ -1445,7 +1469,7 @@ cudaError_t collapse_write(cudaStream_t s, int width, const float4* binary_nodes
     CollapseScratch c((char*)scratch, n_binary, sah_dp);
     CollapseTree& t = c.a.tree[width == 8];
     t.dp.w = area_w;
-    const unsigned blocks = (unsigned)((n_wide + kCollapseThreads - 1) / kCollapseThreads);
+    const unsigned blocks = (unsigned)((n_wide * width + kCollapseThreads - 1) / kCollapseThreads);
     if (width == 8)
         k_collapse_nodes<8><<<blocks, kCollapseThreads, 0, s>>>(binary_nodes, (int)n_wide, t.root, t.first, nodes, t.dp,
                                                                 sah_dp ? 1 : 0);
