@@ -349,6 +349,13 @@ constexpr int kAdjBlocks = 1024;
 // rounding shift) and writes those gradients; block 0 sums the per-block loss
 // partials in block order.  Every step is a deterministic function of the
 // tape and the grid size, so the result is bit-reproducible run to run.
+//
+// What bounds it at 1M beams (15 MB, two chunks a block): not the bytes but
+// the chain of phases, about 6 us until the chunks are in and added and as
+// much again for the block's totals, the wait and the merge.  So every thread
+// reads the warps' maxima itself instead of waiting for one that does, the
+// loss and the counts are added beside the rest, and the merge's sub-groups
+// meet by shuffles: a zeroed call of the adjoint 27.3 -> 25.6 us.
 
 constexpr int kOneThreads = 512;
 constexpr int kOneBPT = 4;                          // beams per thread per chunk (one per warp step)
@@ -503,10 +510,7 @@ struct Acc32 {
 __device__ __forceinline__ void grid_arrive(unsigned long long* arrivals)
 {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(arrivals, 1ull);
-    }
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrivals) : "memory");
 }
 
 __device__ __forceinline__ bool grid_wait_for(unsigned long long* arrivals, unsigned long long target, int* status,
@@ -515,7 +519,10 @@ __device__ __forceinline__ bool grid_wait_for(unsigned long long* arrivals, unsi
     if (threadIdx.x == 0) {
         int ok = 1;
         const uint64_t t0 = adj_global_ns();
-        while (*(volatile unsigned long long*)arrivals < target) {
+        for (;;) {
+            unsigned long long seen;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(arrivals) : "memory");
+            if (seen >= target) break;
             if (adj_global_ns() - t0 > wait_ns) {
                 raise_status(status, ST_TIMEOUT);
                 ok = 0;
@@ -523,11 +530,37 @@ __device__ __forceinline__ bool grid_wait_for(unsigned long long* arrivals, unsi
             }
             __nanosleep(32);
         }
-        __threadfence();
         *s_flag = ok;
     }
     __syncthreads();
     return *s_flag != 0;
+}
+
+// largest of the lanes' values (none negative or NaN: the bits order like the values)
+__device__ __forceinline__ float warp_max(float x)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+}
+
+// largest of what the warps left, by every thread for itself
+__device__ __forceinline__ float warps_max(const float* s)
+{
+    float m = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kOneWarps; w += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(&s[w]);
+        m = fmaxf(fmaxf(m, fmaxf(q.x, q.y)), fmaxf(q.z, q.w));
+    }
+    return m;
+}
+
+// sum of the lanes' counts (beams of a tape: below 2^54), 27 bits at a time
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long x)
+{
+    constexpr unsigned kLow = (1u << 27) - 1u;
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & kLow);
+    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 27));
+    return ((unsigned long long)hi << 27) + lo;
 }
 
 template <bool kTma>
@@ -544,7 +577,6 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
     __shared__ double s_red[kOneThreads];
     __shared__ unsigned long long s_cnt[kOneWarps];
     __shared__ int s_flag;
-    __shared__ float s_gmax;
     __shared__ int s_sh[kOneMaxGrid];  // every block's fixed-point shift
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -687,7 +719,7 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
             loss32 = __fmaf_rn(res, res, loss32);
             ++cnt;
         }
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mx = warp_max(mx);
         if (lane == 0) s_wmax[k & 1][warp] = mx;
         // every thread has read this chunk's stage and published its maximum
         if (__syncthreads_or(!ok)) {
@@ -702,12 +734,7 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
             issue(issued);
             ++issued;
         }
-        float cm = 0.0f;
-#pragma unroll
-        for (int w = 0; w < kOneWarps; w += 4) {
-            const float4 q = *reinterpret_cast<const float4*>(&s_wmax[k & 1][w]);
-            cm = fmaxf(fmaxf(cm, fmaxf(q.x, q.y)), fmaxf(q.z, q.w));
-        }
+        const float cm = warps_max(s_wmax[k & 1]);
         if (cm > blk_max) {
             const int nsh = one_shift(cm, L);
             if (nsh < sh && blk_max > 0.0f) {
@@ -757,46 +784,41 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
 
     // ---- this block's gain-term maximum, loss partial (fixed order), beam count:
     // FP32 within a warp (a fixed shuffle tree), FP64 across warps
-    float gmx = fabsf(gain32);
+    // (every thread finds the maximum itself; one thread adds the partials up
+    // beside the rest)
+    const float gmx = warp_max(fmaxf(fabsf(gain32), 0.0f));
     float l = loss32;
-    unsigned c = cnt;
-    for (int o = 16; o > 0; o >>= 1) {
-        gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
-        l += __shfl_down_sync(0xffffffffu, l, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
+    const unsigned c = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) {
         s_red[warp] = (double)l;
         s_cnt[warp] = c;
         s_wmax[0][warp] = gmx;
     }
     __syncthreads();
-    if (tid == 0) {
+    if (tid == kOneThreads - 1) {
         double t = 0.0;
         unsigned long long ct = 0;
-        float gm = 0.0f;
         for (int w = 0; w < kOneWarps; ++w) {
             t += s_red[w];
             ct += s_cnt[w];
-            gm = fmaxf(gm, s_wmax[0][w]);
         }
-        s_gmax = gm;
         a.blk_loss[blk] = t;
         a.blk_n[blk] = ct;
     }
-    __syncthreads();
+    const float block_gmax = warps_max(s_wmax[0]);
     // the threads' gain sums join the fixed-point sums: widen the scale first
     // if one of them is larger than every term seen
-    if (s_gmax > blk_max && !failed) {
-        const int nsh = one_shift(s_gmax, L);
+    if (block_gmax > blk_max && !failed) {
+        const int nsh = one_shift(block_gmax, L);
         if (nsh < sh && blk_max > 0.0f) {
             const int dd = sh - nsh;
             for (int j = tid; j < a.n_acc; j += kOneThreads) acc.set(j, round_shift(acc.get(j), dd));
+            __syncthreads();
         }
         if (nsh < sh) sh = nsh;
-        blk_max = s_gmax;
+        blk_max = block_gmax;
     }
-    __syncthreads();
     if (blk_max > 0.0f) {
         long long gq = fixed_of(gain32, ldexpf(1.0f, sh));
         for (int o = 16; o > 0; o >>= 1) gq += __shfl_xor_sync(0xffffffffu, gq, o);
@@ -863,43 +885,31 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
             N += __ldcg(&a.blk_n[j]);
             s_sh[j] = __ldcg(&a.blk_sh[j]);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
-            N += __shfl_xor_sync(0xffffffffu, N, o);
-        }
+        gm = warp_max(gm);
+        N = warp_sum(N);
         if (lane == 0) {
             s_wmax[1][warp] = gm;
             s_cnt[warp] = N;
         }
-        __syncthreads();
-        if (tid == 0) {
-            float g2 = 0.0f;
-            unsigned long long n2 = 0;
-            for (int w = 0; w < kOneWarps; ++w) {
-                g2 = fmaxf(g2, s_wmax[1][w]);
-                n2 += s_cnt[w];
-            }
-            s_gmax = g2;
-            s_cnt[0] = n2;
-        }
-        __syncthreads();
     }
-    const float gmax = s_gmax;
-    const unsigned long long N = s_cnt[0];
+    // block 0's last warp adds the loss partials in a fixed order (lane l takes
+    // blocks l, l + 32, ..., then a fixed shuffle tree)
+    double loss = 0.0;
+    const bool writes_loss = blk == 0 && warp == kOneWarps - 1 && a.loss;
+    if (writes_loss) {
+        for (int j = lane; j < G; j += 32) loss += __ldcg(&a.blk_loss[j]);
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
+    }
+    __syncthreads();
+    const float gmax = warps_max(s_wmax[1]);
+    const unsigned long long N = warp_sum(lane < kOneWarps ? s_cnt[lane] : 0ull);
     const int S = one_shift(gmax, n);
-    // block 0's last warp writes the loss: the partials in a fixed order (lane
-    // l takes blocks l, l + 32, ..., then a fixed shuffle tree)
     if (blk == 0 && tid == 0 && a.n_used) *a.n_used = N;
-    if (blk == 0 && warp == kOneWarps - 1 && a.loss) {
-        double t = 0.0;
-        for (int j = lane; j < G; j += 32) t += __ldcg(&a.blk_loss[j]);
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) *a.loss = a.mse ? (float)(N ? t / (double)N : 0.0) : 0.0f;
-    }
+    if (writes_loss && lane == 0) *a.loss = a.mse ? (float)(N ? loss / (double)N : 0.0) : 0.0f;
     // each block sums every row over its slice of the entries, each row
     // shifted from its block's scale to the common one (a rounding shift, as
     // the block would have made), and writes those gradients; the warps' and
-    // sub-groups' sums meet in shared memory (integer sums: the order is free)
+    // sub-groups' sums meet by shuffles and in shared memory (integer sums: the order is free)
     if (!failed && gmax > 0.0f) {
         const float inv_scale = ldexpf(1.0f, -S);  // exact: a power of two
         const float norm = a.mse ? (N ? __frcp_rn((float)N) : 0.0f) : 1.0f;
@@ -922,12 +932,19 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
                     if (sub < R && r < G) t += round_shift(v[u], s_sh[r] - S);
                 }
             }
-            s_part[warp * 32 + lane] = t;
+            // the sub-groups' sums to the first
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                if (o >= R) continue;
+                const long long up = __shfl_down_sync(0xffffffffu, t, (unsigned)(o * P));
+                if (sub + o < R) t += up;
+            }
+            if (lane < P) s_part[warp * 32 + lane] = t;
             __syncthreads();
             if (warp == 0 && lane < P) {
                 long long tot = 0;
-                for (int w = 0; w < kOneWarps; ++w)
-                    for (int q = 0; q < R; ++q) tot += s_part[w * 32 + q * P + lane];
+#pragma unroll
+                for (int w = 0; w < kOneWarps; ++w) tot += s_part[w * 32 + lane];
                 const float v = __fmul_rn(__fmul_rn(__ll2float_rn(tot), inv_scale), norm);
                 const int jj = e0 + lane;
                 if (jj < a.n_acc - 1) {
@@ -936,7 +953,7 @@ __global__ void __launch_bounds__(kOneThreads, 2) k_adj_onepass(const __grid_con
                     *a.grad_gain = (e0 == j0 ? g_prev : *a.grad_gain) + v;
                 }
             }
-            __syncthreads();
+            if (e0 + 32 < j1) __syncthreads();  // the next piece's sums take these's place
         }
     }
 }
