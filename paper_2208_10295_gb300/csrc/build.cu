@@ -426,9 +426,7 @@ __device__ bool build_meet(MeetPlace* at, unsigned blocks, unsigned& met, int* s
     ++met;
     bool ok = true;
     if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&at->arrived, 1u) + 1u == met * blocks) {
-            __threadfence();
+        if (arrive(&at->arrived) + 1u == met * blocks) {
             st_release(&at->released, met);
         } else {
             ok = build_spin(status, [&] { return ld_acquire(&at->released) >= met; });
@@ -735,11 +733,9 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
         bool last = false;
         if (tid == 0) {
             __stcg(&a.total[blockIdx.x], ((mine >> 32) << 28) | (mine & 0xFFFFFFFull));
-            __threadfence();
-            last = atomicAdd(&at->arrived, 1u) + 1u == (g.round + 1u) * blocks;
+            last = arrive(&at->arrived) + 1u == (g.round + 1u) * blocks;
         }
         if (__syncthreads_or(last)) {
-            __threadfence();
             const unsigned long long v = tid < (int)blocks ? __ldcg(&a.total[tid]) : 0ull;
             unsigned long long sum;
             const unsigned long long x = block_prefix<kPlocThreads>(v, sum);
