@@ -90,3 +90,127 @@ def test_leaves_in_morton_order(L, n):
         scene.free()
     finally:
         L.set_build_options(method=1)
+
+
+def _integer_triangles(n, seed):
+    """Corners on an integer grid: every area of the build is a whole number below 2^24, exact in FP32."""
+    rng = np.random.default_rng(seed)
+    at = rng.integers(0, 1000, (n, 1, 3))
+    verts = (at + rng.integers(0, 20, (n, 3, 3))).astype(np.float32).reshape(-1, 3)
+    return verts, np.arange(3 * n, dtype=np.uint32).reshape(n, 3)
+
+
+def _ploc_children(lo, hi, radius):
+    """Children of every node of the clustering: nearest neighbours within `radius` (ties to the lower position),
+    mutual pairs merge at the lower position, ids count down from n - 2."""
+    n = len(lo)
+    ref, child, top = ~np.arange(n, dtype=np.int32), np.zeros((n - 1, 2), np.int32), n - 2
+    while len(ref) > 1:
+        m = len(ref)
+        best_d, best = np.full(m, np.inf, np.float32), np.full(m, -1)
+        for off in [o for o in range(-radius, radius + 1) if o and abs(o) < m]:
+            e = slice(max(0, -off), m - max(0, off))
+            o = slice(max(0, off), m + min(0, off))
+            d = np.maximum(hi[e], hi[o]) - np.minimum(lo[e], lo[o])
+            area = d[:, 0] * d[:, 1] + d[:, 1] * d[:, 2] + d[:, 2] * d[:, 0]
+            nearer = area < best_d[e]
+            best_d[e] = np.where(nearer, area, best_d[e])
+            best[e] = np.where(nearer, np.arange(m)[o], best[e])
+        mutual = best[best] == np.arange(m)
+        left = np.nonzero(mutual & (np.arange(m) < best))[0]
+        right = best[left]
+        assert len(left)
+        ids = top - np.arange(len(left), dtype=np.int32)
+        child[ids, 0], child[ids, 1] = ref[left], ref[right]
+        lo[left], hi[left] = np.minimum(lo[left], lo[right]), np.maximum(hi[left], hi[right])
+        ref[left] = ids
+        stay = np.ones(m, bool)
+        stay[right] = False
+        lo, hi, ref, top = lo[stay], hi[stay], ref[stay], top - len(left)
+    return child
+
+
+@pytest.mark.parametrize("n,radius", [(2, 16), (3, 16), (33, 16), (511, 16), (512, 16), (513, 16), (1024, 16),
+                                      (4864, 16), (4865, 16), (14593, 16), (34049, 16), (72961, 16), (150784, 16),
+                                      (150785, 16), (400, 1), (5000, 1), (200000, 1), (513, 5), (90001, 5), (600, 64),
+                                      (19457, 64), (58369, 64), (140000, 64)])
+def test_clustering_at_its_widths(L, n, radius):
+    """One block alone, 8 / 4 / 2 / 1 lanes a cluster, two clusters a thread, several tiles a block (152 SMs)."""
+    verts, tris = _integer_triangles(n, n + radius)
+    try:
+        L.set_build_options(method=1, ploc_radius=radius)
+        scene = L.build_scene(verts, tris)
+        nodes, leaf = scene.export()
+        v = verts[tris[leaf]]
+        assert np.array_equal(nodes[:, 12:14].view(np.int32), _ploc_children(v.min(1), v.max(1), radius))
+        scene.free()
+    finally:
+        L.set_build_options(method=1, ploc_radius=16)
+
+
+def _wide_children(nodes, width):
+    """Wide nodes breadth-first, each the binary references of its children: the one of largest area is opened (ties to
+    the first) until there are `width` or only triangles; internal ones first."""
+    child = nodes[:, 12:14].view(np.int32)
+    b = nodes[:, :12].astype(np.float64)
+    lo = np.stack([b[:, [0, 4]], b[:, [2, 6]], b[:, [8, 10]]], -1)
+    hi = np.stack([b[:, [1, 5]], b[:, [3, 7]], b[:, [9, 11]]], -1)
+    d = hi - lo
+    area = d[..., 0] * d[..., 1] + d[..., 1] * d[..., 2] + d[..., 2] * d[..., 0]
+    out, frontier = [], [0]
+    while frontier:
+        below = []
+        for node in frontier:
+            kids = [(child[node, s], area[node, s]) for s in (0, 1)]
+            while len(kids) < width and any(r >= 0 for r, _ in kids):
+                at = max((k for k in range(len(kids)) if kids[k][0] >= 0), key=lambda k: (kids[k][1], -k))
+                o = kids[at][0]
+                kids[at] = (child[o, 0], area[o, 0])
+                kids.append((child[o, 1], area[o, 1]))
+            refs = [int(r) for r, _ in kids]
+            inner = [r for r in refs if r >= 0]
+            out.append((inner, [r for r in refs if r < 0]))
+            below += inner
+        frontier = below
+    return out
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 8, 9, 33, 257, 1025, 1100, 5000])
+def test_wide_nodes(L, n):
+    """Children and their order by the largest-area rule, and the layout of both rules' trees."""
+    from test_gpu_parity import _wide_tree_invariants
+    verts, tris = _integer_triangles(n, 3 * n)
+    try:
+        for collapse in (0, 1):
+            L.set_build_options(method=1, collapse=collapse)
+            scene = L.build_scene(verts, tris)
+            nodes, leaf = scene.export()
+            v = verts[tris[leaf]]
+            for width in (4, 8):
+                got = scene.export_wide(width)
+                _wide_tree_invariants(got, width, n, v.min(1), v.max(1))
+                if collapse == 0:
+                    code = got.reshape(len(got), -1, 4)[:, 6 * (width // 4):7 * (width // 4)].reshape(len(got), width)
+                    first = 1
+                    want = np.zeros((len(got), width), np.int32)
+                    for i, (inner, leaves) in enumerate(_wide_children(nodes, width)):
+                        row = list(range(first, first + len(inner))) + leaves
+                        want[i, :len(row)] = row
+                        first += len(inner)
+                    assert np.array_equal(code.view(np.int32), want)
+            scene.free()
+    finally:
+        L.set_build_options(method=1, collapse=0)
+
+
+def test_scenes_come_and_go(L):
+    """The arrays of freed scenes serve the next ones: scenes of changing sizes, freed out of order, stay whole."""
+    kept = []
+    for k, n in enumerate([5000, 33, 70001, 2, 4097, 5000]):
+        verts, tris = _random_triangles(n, 100 + k)
+        kept.append((L.build_scene(verts, tris), verts, tris))
+        if k % 2:
+            kept.pop(0)[0].free()
+    for scene, verts, tris in kept:
+        _check_binary_tree(*scene.export(), verts, tris)
+        scene.free()
