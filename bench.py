@@ -64,31 +64,31 @@ POINT_BYTES = 12 + 4 + 4 + 12 + 2 + 4 + 4 + 4   # xyz, range, intensity, normal,
 # the cast kernel as the roofline times it (cfg1 frame, dense valid flags out,
 # L2 flushed before the launch), from one ncu capture, with the digest of the
 # kernel sources the capture ran.  Reported only while the sources still match.
-NCU_TRAFFIC = {"sources": "43cc999e0fe54cea", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
-               "bytes": 9_744_640, "l2_bytes": 3_380_907 * 32,
-               "l1_global_load_bytes": 6_591_193 * 32}   # profiles/k_cast_cfg1_ncu_full.md
+NCU_TRAFFIC = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
+               "bytes": 9_704_192 + 58_368, "l2_bytes": 3_410_835 * 32,
+               "l1_global_load_bytes": 6_629_948 * 32}   # profiles/k_cast_cfg1_ncu_full.md
 # Binding-unit fractions of the same capture (ncu --set full of one launch):
 # L1/TEX throughput, issue-active and SM-active shares.
-NCU_UNITS = {"l1tex_throughput_pct": 41.1, "issue_active_pct": 43.4, "sm_active_pct": 71.0}
+NCU_UNITS = {"l1tex_throughput_pct": 45.6, "issue_active_pct": 42.3, "sm_active_pct": 71.1}
 # FP32 work of one launch of the cast kernel from ncu's SASS instruction
 # counters (sm__sass_thread_inst_executed_op_{ffma,fadd,fmul,ffma2,fadd2,fmul2,
 # fp32}_pred_on), FLOPs = 2 ffma + fadd + fmul + 4 ffma2 + 2 fadd2 + 2 fmul2 +
 # the remaining FP32 instructions (min/max, compares) once each.
-NCU_FP32 = {"sources": "43cc999e0fe54cea", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
-            "fp32_flops": 497_878_528, "fp32_ops": 476_442_679,
-            "counters": {"ffma": 21_435_849, "fadd": 10_460_945, "fmul": 33_010_988, "ffma2": 0,
-                         "fadd2": 68_563_704, "fmul2": 68_563_704, "fp32_all": 339_315_271}}
+NCU_FP32 = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
+            "fp32_flops": 499_329_365, "fp32_ops": 339_857_714,
+            "counters": {"ffma": 22_224_867, "fadd": 12_038_981, "fmul": 34_606_334, "ffma2": 68_623_392,
+                         "fadd2": 0, "fmul2": 0, "fp32_all": 271_234_322}}
 # profiles/k_cast_cfg1_fp32_counts.md
 # Binding-unit fractions of one city frame launch (ncu --set full,
 # profiles/k_cast_city_ncu_full.md), with the sources and tree it ran
-NCU_CITY_UNITS = {"sources": "43cc999e0fe54cea", "tree": dict(treelet_rounds=8, area_weight=(1.0, 1.0, 0.35)),
+NCU_CITY_UNITS = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=8, area_weight=(1.0, 1.0, 0.35)),
                   "kernel": "k_cast<0, 4, 2>",
-                  "issue_active_pct": 74.8, "l1tex_throughput_pct": 62.9, "fma_pipe_pct": 42.7, "alu_pipe_pct": 53.5}
+                  "issue_active_pct": 76.2, "l1tex_throughput_pct": 69.8, "fma_pipe_pct": 32.0, "alu_pipe_pct": 60.7}
 KERNEL_SOURCES = ("cast.cu", "shade.cuh", "trace.cuh", "common.cuh", "philox.cuh")
 # DRAM traffic (read + write) of one launch of the one-pass adjoint on the
 # 16-frame tape, from one ncu capture (profiles/k_adj_cfg3_ncu_full.md),
 # reported while adjoint.cu still has the captured digest
-ADJ_TRAFFIC = {"sources": "0d4c79dc0d5a7f66", "bytes": 67_204_352 + 2_014_464}
+ADJ_TRAFFIC = {"sources": "d296c3242e5507ca", "bytes": 67_207_680 + 1_036_288}
 
 
 def kernel_digest():
@@ -472,7 +472,7 @@ def run_ours(args, rank, world, local_rank):
                    captured_launch)
     traffic = NCU_TRAFFIC["bytes"] if same_kernel else None
     sm_mhz = (clocks or {}).get("sm_mhz") or peaks.get("clocks_under_load", {}).get("sm_mhz_median", 1455.0)
-    # FP32 ops per child box of a fetched node: 6 slab subtracts + 6 multiplies, 3 max (entry, with t_eps),
+    # FP32 ops per child box of a fetched node: 6 slab FMAs (two each), 3 max (entry, with t_eps),
     # 2 min (exit), the far-scale multiply, the min with the best hit and the compare = 20; a node holds
     # node_bytes / 32 children (2, 4 or 8); 40 per watertight triangle test
     flops = counters["node_visits"] * (counters["node_bytes"] // 32) * 20 + counters["tri_tests"] * 40
@@ -537,7 +537,7 @@ def run_ours(args, rank, world, local_rank):
                                        if fp_probe.get("sm_mhz") else None),
                 "ops_per_launch_alg": flops, "ops_per_launch_ncu": NCU_FP32["fp32_ops"] if ncu_ok else None,
                 "ops": "alg: 20 FP32 ops per child box of a fetched node, 40 per triangle test (from the "
-                       "source, each operation once); ncu: FP32 thread instructions of one captured launch "
+                       "source, an FMA as two); ncu: FP32 thread instructions of one captured launch "
                        "(sm__sass_thread_inst_executed_op_*_pred_on), each lane operation once (ops) or with "
                        "FMAs and packed pairs counted as two (flops, the unit of the measured peak)"},
         "clocks": clocks,
