@@ -223,6 +223,11 @@ cudaError_t scene_alloc(lidar_ctx* c, void** p, size_t bytes)
     }
     if (!c->pool) return dev_alloc(p, bytes);
     *p = nullptr;
+    // a build synchronises, which a capture cannot hold: refused here, as
+    // cudaMalloc would refuse it, and not turned into a node of the graph
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+        return cudaErrorStreamCaptureUnsupported;
     if (alloc_fault()) return cudaErrorMemoryAllocation;
     return cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
 }
