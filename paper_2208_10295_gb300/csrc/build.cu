@@ -1217,46 +1217,70 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
         const int tiles = (n + T - 1) / T;
         const int per = (tiles + (int)of - 1) / (int)of;
         const int t0 = min((int)me * per, tiles), t1 = min(t0 + per, tiles);
+        const bool shared = tiles > 1 || of > 1;
+        int ref[W], count = 0, internal = 0, below = 0;  // this thread's node of the last tile
+        unsigned before = 0, sum = 0;
         for (int t = t0; t < t1; ++t) {
             const int i = t * T + tid;
-            int internal = 0;
+            count = internal = 0;
             if (i < n) {
-                int ref[W], count;
                 const int slot = base + i;
                 internal = gather_refs<W>(a.bn, slot ? __ldcg(&c.root[slot]) : 0, c.dp, a.use_dp, ref, count);
-                int m = 0;
+                below = (slot ? __ldcg(&c.pushes[slot]) : 0) + (internal > 0 ? internal - 1 : 0);
+                need = max(need, below);
+                if (per > 1) {
+                    int m = 0;
+#pragma unroll
+                    for (int k = 0; k < W; ++k)
+                        if (k < count && ref[k] >= 0) __stcg(&c.kids[(int64_t)i * W + m++], ref[k]);
+                    __stcg(&c.first[slot], internal);
+                }
+            }
+            before = block_prefix<T>((unsigned)internal, sum);
+            if (shared && tid == 0) __stcg(&c.total[t], sum);
+        }
+        // internal children of the tiles before this block's, and of all
+        unsigned at = 0, next = sum;
+        if (shared) {
+            if (!build_meet(c.place, of, met, a.status)) return false;
+            unsigned mine = 0, all = 0;
+            for (int t = tid; t < tiles; t += T) {
+                const unsigned v = __ldcg(&c.total[t]);
+                all += v;
+                if (t < t0) mine += v;
+            }
+            block_prefix<T>(mine, at);
+            block_prefix<T>(all, next);
+        }
+        if (per == 1) {
+            // the thread still holds its node's children (listed in memory in
+            // between, and a lone block's sum too, a rebuild and cast took 317 us
+            // at 770 triangles and 1,358 us at 1M; 296 and 1,338 us so)
+            const int slot = base + t0 * T + tid;
+            if (count > 0) {
+                int off = base + n + (int)(at + before);
+                __stcg(&c.first[slot], internal > 0 ? off : 0);
 #pragma unroll
                 for (int k = 0; k < W; ++k)
-                    if (k < count && ref[k] >= 0) __stcg(&c.kids[(int64_t)i * W + m++], ref[k]);
-                __stcg(&c.first[slot], internal);
-                need = max(need, (slot ? __ldcg(&c.pushes[slot]) : 0) + (internal > 0 ? internal - 1 : 0));
+                    if (k < count && ref[k] >= 0) {
+                        __stcg(&c.root[off], ref[k]);
+                        __stcg(&c.pushes[off], below);
+                        ++off;
+                    }
             }
-            unsigned sum;
-            block_prefix<T>((unsigned)internal, sum);
-            if (tid == 0) __stcg(&c.total[t], sum);
-        }
-        if (!build_meet(c.place, of, met, a.status)) return false;
-        unsigned before = 0, all = 0;
-        for (int t = tid; t < tiles; t += T) {
-            const unsigned v = __ldcg(&c.total[t]);
-            all += v;
-            if (t < t0) before += v;
-        }
-        unsigned at, next;
-        block_prefix<T>(before, at);
-        block_prefix<T>(all, next);
-        for (int t = t0; t < t1; ++t) {
-            const int i = t * T + tid, slot = base + i;
-            const int internal = i < n ? __ldcg(&c.first[slot]) : 0;
-            unsigned sum;
-            const int off = base + n + (int)(at + block_prefix<T>((unsigned)internal, sum));
-            at += sum;
-            if (i >= n) continue;
-            const int below = (slot ? __ldcg(&c.pushes[slot]) : 0) + (internal > 0 ? internal - 1 : 0);
-            __stcg(&c.first[slot], internal > 0 ? off : 0);
-            for (int k = 0; k < internal; ++k) {
-                __stcg(&c.root[off + k], __ldcg(&c.kids[(int64_t)i * W + k]));
-                __stcg(&c.pushes[off + k], below);
+        } else {
+            for (int t = t0; t < t1; ++t) {
+                const int i = t * T + tid, slot = base + i;
+                internal = i < n ? __ldcg(&c.first[slot]) : 0;
+                const int off = base + n + (int)(at + block_prefix<T>((unsigned)internal, sum));
+                at += sum;
+                if (i >= n) continue;
+                below = (slot ? __ldcg(&c.pushes[slot]) : 0) + (internal > 0 ? internal - 1 : 0);
+                __stcg(&c.first[slot], internal > 0 ? off : 0);
+                for (int k = 0; k < internal; ++k) {
+                    __stcg(&c.root[off + k], __ldcg(&c.kids[(int64_t)i * W + k]));
+                    __stcg(&c.pushes[off + k], below);
+                }
             }
         }
         base += n;

@@ -130,10 +130,11 @@ def _ploc_children(lo, hi, radius):
     return child
 
 
-@pytest.mark.parametrize("n,radius", [(2, 16), (3, 16), (33, 16), (511, 16), (512, 16), (513, 16), (1024, 16),
-                                      (4864, 16), (4865, 16), (14593, 16), (34049, 16), (72961, 16), (150784, 16),
-                                      (150785, 16), (400, 1), (5000, 1), (200000, 1), (513, 5), (90001, 5), (600, 64),
-                                      (19457, 64), (58369, 64), (140000, 64)])
+@pytest.mark.parametrize("n,radius", [(2, 16), (3, 16), (33, 16), (511, 16), (512, 16), (513, 16), (1023, 16),
+                                      (1024, 16), (1025, 16), (4864, 16), (4865, 16), (14593, 16), (34049, 16),
+                                      (72961, 16), (150784, 16), (150785, 16), (400, 1), (5000, 1), (200000, 1),
+                                      (513, 5), (1000, 5), (90001, 5), (600, 64), (1024, 64), (19457, 64),
+                                      (58369, 64), (140000, 64)])
 def test_clustering_at_its_widths(L, n, radius):
     """One block alone, 8 / 4 / 2 / 1 lanes a cluster, two clusters a thread, several tiles a block (152 SMs)."""
     verts, tris = _integer_triangles(n, n + radius)
