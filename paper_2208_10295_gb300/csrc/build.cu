@@ -817,7 +817,7 @@ constexpr size_t kPlocShared = sizeof(PlocShared) + kPlocWide * kPlocThreads * s
 // round's chain (an exchange of counts and a meeting, ~5 us, a search) and, in
 // the first rounds, the 2 radius box unions per cluster (~30 issue slots each,
 // half of them min / max).  1M triangles: 0.69 ms with one cluster a thread,
-// everything through L2 and the blocks polling one counter; 0.58 ms so.  Four
+// everything through L2 and the blocks polling one counter; 0.56 ms so.  Four
 // clusters a thread, or 1,024 threads, take as long: the searches are bound
 // by issue, the rest by the chain.
 __global__ void __launch_bounds__(kPlocThreads, 1) k_ploc(PlocArgs a)
@@ -1909,8 +1909,9 @@ __device__ int treelet_node(const TreeletArgs& a, int node, TreeletShared& t, in
 // One warp a block: warps end at very different times (most lanes stop after a
 // few steps, a few climb to the root), and a block's slot is only free when its
 // last warp ends.  16 a SM leaves 128 registers, without spills (0.65M
-// triangles, eight rounds, the whole build and a cast: 11.0 ms; four-warp
-// blocks 11.4 ms; 80 registers and 24 warps 11.3 ms, with spills).
+// triangles, eight rounds, the whole build and a cast: 5.54 ms; with spills,
+// 18 and 20 a SM 6.0 ms, 24 and 28 6.4 and 6.5 ms; four-warp blocks, when the
+// rest took longer, 11.4 ms against 11.0).
 constexpr int kTreeletThreads = 32;
 constexpr int kTreeletBlocks = 16;
 
@@ -1953,7 +1954,9 @@ __global__ void __launch_bounds__(kBuildThreads) k_treelet_paths(TreeletArgs a)
 // treelet with its program in local memory 9.4 ms a round; by a warp 1.2 ms;
 // with the treelets whose subtree is unchanged kept unseen 1.2, 0.88, 0.64,
 // 0.51, 0.41, 0.35, 0.31, 0.30 ms; climbing only where something was rewritten
-// 1.2, 0.85, 0.62, 0.43, 0.35, 0.30, 0.24, 0.25 ms.
+// and with one acquire-release arrival a level 1.14, 0.83, 0.60, 0.42, 0.32,
+// 0.30, 0.25, 0.24 ms.  A stride between a warp's nodes, fewer lanes or more
+// nodes a warp all took longer: neighbours share the climb.
 __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_round(TreeletArgs a)
 {
     __shared__ TreeletShared s_t[kTreeletThreads / 32];
