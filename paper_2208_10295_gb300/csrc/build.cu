@@ -10,6 +10,7 @@
 //      writes both child boxes (exact FP32 min/max, no rounding) and the node
 //      height; the first stops.  The root height bounds the traversal stack.
 #include "common.cuh"
+#include "ploc_counts.h"
 
 #include <algorithm>
 #include <type_traits>
@@ -480,8 +481,8 @@ struct PlocArgs {
     int n;
     float4* cluster[2];           // [2 n] each: lo, ref bits; hi, height bits (the rounds alternate)
     int* mate;                    // [n] >= 0: merges with that later position; -1: stays; -2: merged away
-    // per block: its merges << 28 | clusters that stay; and, in a sector of its
-    // own, those before it and of all, each with the round's tag << 56
+    // per block: its counts (ploc_counts.h); and, in a sector of its own, those
+    // before it and of all, each with the round's tag
     unsigned long long* total;    // [kPlocMaxBlocks]
     unsigned long long* answer;   // [kPlocMaxBlocks][4]
     float4* nodes;
@@ -677,7 +678,7 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
     const int first = K > 1 ? K * tid : tid / lanes;  // this thread's first cluster of those held
     int mate[K];                                      // of the last tile's
     unsigned place = 0, count;                        // merges << 16 | stays before this thread's, and of the tile
-    unsigned long long mine = 0;                      // merges << 32 | stays of the block's tiles
+    unsigned long long mine = 0;                      // counts of the block's tiles
 #pragma unroll
     for (int i = 0; i < K; ++i) mate[i] = -2;
     for (int t = t0; t < t1; ++t) {
@@ -720,7 +721,7 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
             if (mate[i] != -2) v += mate[i] >= 0 ? 0x10001u : 1u;
         }
         place = block_prefix<kPlocThreads>(v, count);
-        mine += ((unsigned long long)(count >> 16) << 32) | (count & 0xFFFFu);
+        mine += ploc_counts(count >> 16, count & 0xFFFFu);
     }
     // merges and stays of the blocks before, and of all
     unsigned long long before = 0;
@@ -728,11 +729,10 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
     if (blocks > 1) {
         // every block leaves its counts and arrives; the last one sums them up
         // and answers each in its own sector
-        const unsigned long long tag = (unsigned long long)(g.round % 200u + 1u) << 56;
         MeetPlace* at = a.place + 1;
         bool last = false;
         if (tid == 0) {
-            __stcg(&a.total[blockIdx.x], ((mine >> 32) << 28) | (mine & 0xFFFFFFFull));
+            __stcg(&a.total[blockIdx.x], mine);
             last = arrive(&at->arrived) + 1u == (g.round + 1u) * blocks;
         }
         if (__syncthreads_or(last)) {
@@ -740,8 +740,8 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
             unsigned long long sum;
             const unsigned long long x = block_prefix<kPlocThreads>(v, sum);
             if (tid < (int)blocks) {
-                *(volatile unsigned long long*)&a.answer[4 * tid] = tag | x;
-                *(volatile unsigned long long*)&a.answer[4 * tid + 1] = tag | sum;
+                *(volatile unsigned long long*)&a.answer[4 * tid] = ploc_tagged(x, g.round);
+                *(volatile unsigned long long*)&a.answer[4 * tid + 1] = ploc_tagged(sum, g.round);
             }
         }
         bool ok = true;
@@ -751,16 +751,16 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
             ok = build_spin(a.status, [&] {
                 x = mine_at[0];
                 y = mine_at[1];
-                return (x >> 56) == (tag >> 56) && (y >> 56) == (tag >> 56);
+                return ploc_is_of(x, g.round) && ploc_is_of(y, g.round);
             });
-            s_sum[0] = x;
-            s_sum[1] = y;
+            s_sum[0] = ploc_untagged(x);
+            s_sum[1] = ploc_untagged(y);
         }
         if (!__syncthreads_and(ok)) return false;
-        before = ((s_sum[0] >> 28 & 0xFFFFFFFull) << 32) | (s_sum[0] & 0xFFFFFFFull);
-        all = ((s_sum[1] >> 28 & 0xFFFFFFFull) << 32) | (s_sum[1] & 0xFFFFFFFull);
+        before = s_sum[0];
+        all = s_sum[1];
     }
-    if ((all >> 32) == 0) return true;
+    if (ploc_merges(all) == 0) return true;
     // the tile at `base`, its boxes in shared memory and its mates in registers
     auto write = [&](int base, unsigned long long at) {
         const int from = base - 2 * halo;
@@ -772,15 +772,15 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
             if (mate[i] >= 0) {
                 float4 rlo, rhi;
                 ploc_get(s_c, mate[i] - from, rlo, rhi);
-                ploc_merge(a, g.id_top - (int)(at >> 32), lo, hi, rlo, rhi);
+                ploc_merge(a, g.id_top - (int)ploc_merges(at), lo, hi, rlo, rhi);
             }
-            const int64_t out = (int64_t)(at & 0xFFFFFFFFull);
+            const int64_t out = ploc_stays(at);
             __stcg(&g.D[2 * out], lo);
             __stcg(&g.D[2 * out + 1], hi);
-            at += mate[i] >= 0 ? (1ull << 32) | 1ull : 1ull;
+            at += ploc_counts(mate[i] >= 0 ? 1u : 0u, 1u);
         }
     };
-    auto wide = [](unsigned v) { return ((unsigned long long)(v >> 16) << 32) | (v & 0xFFFFu); };
+    auto wide = [](unsigned v) { return ploc_counts(v >> 16, v & 0xFFFFu); };
     if (per == 1) {
         write(t0 * T, before + wide(place));
         return true;
@@ -846,10 +846,10 @@ __global__ void __launch_bounds__(kPlocThreads, 1) k_ploc(PlocArgs a)
         if (!(g.lanes ? ploc_round<1>(a, s_c, s_nn, blocks, g, all) : ploc_round<kPlocWide>(a, s_c, s_nn, blocks, g, all)))
             return;
         ++g.round;
-        g.force = (all >> 32) == 0;  // then nothing was written
+        g.force = ploc_merges(all) == 0;  // then nothing was written
         if (!g.force) {
-            g.id_top -= (int)(all >> 32);
-            g.nc = (int)(all & 0xFFFFFFFFull);
+            g.id_top -= (int)ploc_merges(all);
+            g.nc = (int)ploc_stays(all);
             const float4* swap = g.C;
             g.C = g.D;
             g.D = const_cast<float4*>(swap);
