@@ -91,7 +91,8 @@ lidar_status lidar_sync_status(lidar_ctx* ctx);
  * n_tris may be 0 (every beam misses).  The input arrays are only read during
  * the call.  This call synchronises the stream to report build errors
  * (LIDAR_EINVAL for an out-of-range vertex index, LIDAR_ESTACK if the tree is
- * deeper than the traversal stack). */
+ * deeper than the traversal stack, LIDAR_ETIMEOUT if a wait of its kernels ran
+ * out, see lidar_set_wait_limit). */
 lidar_status lidar_scene_build(lidar_ctx* ctx, const float* verts_dev, int64_t n_verts,
                                const uint32_t* tris_dev, int64_t n_tris,
                                const uint16_t* tri_material_dev, const uint32_t* tri_instance_dev,
@@ -583,11 +584,13 @@ lidar_status lidar_get_cast_overlap(lidar_ctx* ctx, int32_t* enable);
 
 /* Limit, in nanoseconds of GPU time (the device's global timer), of every
  * bounded device-side wait in the context's kernels: the grid-wide wait of a
- * cast whose point-cloud scatter runs inside the cast kernel, and the waits of
- * the one-pass adjoint.  A wait that runs out records LIDAR_ETIMEOUT in the
- * status word (read by lidar_sync_status) and its block leaves the kernel
- * without the work after the wait, so that call's outputs past the wait are
- * incomplete; nothing hangs and the context stays usable.  Default
+ * cast whose point-cloud scatter runs inside the cast kernel, the waits of the
+ * one-pass adjoint, and those of a scene build's blocks for one another.  A
+ * wait that runs out records LIDAR_ETIMEOUT in the status word (read by
+ * lidar_sync_status; lidar_scene_build returns it and makes no scene) and its
+ * block leaves the kernel without the work after the wait, so that call's
+ * outputs past the wait are incomplete; nothing hangs and the context stays
+ * usable.  Default
  * 2,000,000,000 (2 s), far beyond any legitimate wait; 0 gives up at the first
  * check that finds the wait unfinished (exercises the timeout path).  Applies
  * to launches made afterwards. */

@@ -303,13 +303,14 @@ size_t build_scratch_bytes(int64_t n)
 }
 
 cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, float4* nodes_out, int* max_height_dev,
-                       int radius, void* scratch, size_t scratch_bytes, AreaW w, int* status, int num_sms, int coop);
+                       int radius, void* scratch, size_t scratch_bytes, AreaW w, int* status, int num_sms, int coop,
+                       uint64_t wait_ns);
 
 cudaError_t build_lbvh(cudaStream_t s, const float* verts, int64_t n_verts, const uint32_t* tris,
                        const uint16_t* mat, const uint32_t* inst, int64_t n, float4* nodes_out,
                        float4* tris_out, uint32_t* leaf_tri_out, int* status, int* max_height_dev,
-                       void* scratch, size_t scratch_bytes, int num_sms, int coop, int method, int radius,
-                       AreaW area_w)
+                       void* scratch, size_t scratch_bytes, int num_sms, int coop, uint64_t wait_ns, int method,
+                       int radius, AreaW area_w)
 {
     if (n == 0) return cudaSuccess;
     if (scratch_bytes < build_scratch_bytes(n)) return cudaErrorInvalidValue;
@@ -341,7 +342,7 @@ cudaError_t build_lbvh(cudaStream_t s, const float* verts, int64_t n_verts, cons
     if (method == 1) {
         // clustering over the Morton-ordered leaves; the sort's buffers are free again
         return build_ploc(s, tris_out, n, nodes_out, max_height_dev, radius, scratch, scratch_bytes, area_w, status,
-                          num_sms, coop);
+                          num_sms, coop, wait_ns);
     }
     const int iblocks = (int)((n - 1 + kBuildThreads - 1) / kBuildThreads);
     k_karras<<<iblocks, kBuildThreads, 0, s>>>(keys, n, nodes_out, parent_node, parent_leaf);
@@ -372,9 +373,6 @@ __device__ __forceinline__ float union_half_area(float4 alo, float4 ahi, float4 
     return w.z * dx * dy + w.x * dy * dz + w.y * dz * dx;
 }
 
-constexpr uint64_t kBuildWaitNs = 2000000000ull;
-
-
 // Where the blocks of a cooperative launch meet: a counter they arrive at and
 // a word, in another line, that the last to arrive sets for the rest to see
 // (both zero before the launch).  With every block reading the counter, or a
@@ -387,18 +385,27 @@ struct MeetPlace {
     unsigned pad1[31];
 };
 
-// Spins until `ready()`.  Bounded: after two seconds ST_TIMEOUT and false.
+// How long a block waits for the others (the context's wait limit), and where
+// it says that it gave up.
+struct BuildWait {
+    int* status;
+    uint64_t ns;
+};
+
+// Spins until `ready()`.  Bounded: after w.ns nanoseconds (0: at once) ST_TIMEOUT
+// and false.  The timer is read every 64th time, so that the reads of what is
+// waited for follow closely.
 template <typename Ready>
-__device__ __forceinline__ bool build_spin(int* status, Ready ready)
+__device__ __forceinline__ bool build_spin(BuildWait w, Ready ready)
 {
     uint64_t t0 = 0;
     for (unsigned it = 1; !ready(); ++it) {
-        if ((it & 63u) != 0u) continue;
+        if ((it & 63u) != 0u && w.ns != 0) continue;
         uint64_t t;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
         if (t0 == 0) t0 = t;
-        if (t - t0 > kBuildWaitNs) {
-            raise_status(status, ST_TIMEOUT);
+        if (t - t0 > w.ns || w.ns == 0) {
+            raise_status(w.status, ST_TIMEOUT);
             return false;
         }
     }
@@ -420,7 +427,7 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v)
 // The `blocks` blocks of a cooperative launch meet for the `met`-th time (this
 // counts it), what each wrote before visible to all after.  One block alone
 // only meets its own threads.  False in every thread when the wait ran out.
-__device__ bool build_meet(MeetPlace* at, unsigned blocks, unsigned& met, int* status)
+__device__ bool build_meet(MeetPlace* at, unsigned blocks, unsigned& met, BuildWait wait)
 {
     __syncthreads();
     if (blocks == 1) return true;
@@ -430,7 +437,7 @@ __device__ bool build_meet(MeetPlace* at, unsigned blocks, unsigned& met, int* s
         if (arrive(&at->arrived) + 1u == met * blocks) {
             st_release(&at->released, met);
         } else {
-            ok = build_spin(status, [&] { return ld_acquire(&at->released) >= met; });
+            ok = build_spin(wait, [&] { return ld_acquire(&at->released) >= met; });
         }
     }
     return __syncthreads_and(ok) != 0;
@@ -490,7 +497,7 @@ struct PlocArgs {
     int radius;
     AreaW w;
     MeetPlace* place;             // the blocks' meetings and exchanges (two), zero before the launch
-    int* status;
+    BuildWait wait;
 };
 
 // Clusters in shared memory: lo x y z, hi x y z, ref bits, height bits.
@@ -748,7 +755,7 @@ __device__ __forceinline__ bool ploc_round(const PlocArgs& a, PlocShared& s_c, i
         if (tid == 0) {
             const volatile unsigned long long* mine_at = a.answer + 4 * blockIdx.x;
             unsigned long long x = 0, y = 0;
-            ok = build_spin(a.status, [&] {
+            ok = build_spin(a.wait, [&] {
                 x = mine_at[0];
                 y = mine_at[1];
                 return ploc_is_of(x, g.round) && ploc_is_of(y, g.round);
@@ -833,7 +840,7 @@ __global__ void __launch_bounds__(kPlocThreads, 1) k_ploc(PlocArgs a)
         __stcg(&a.cluster[0][2 * i], make_float4(b.lo[0], b.lo[1], b.lo[2], __int_as_float(~(int)i)));
         __stcg(&a.cluster[0][2 * i + 1], make_float4(b.hi[0], b.hi[1], b.hi[2], __int_as_float(0)));
     }
-    if (!build_meet(a.place, blocks, met, a.status)) return;
+    if (!build_meet(a.place, blocks, met, a.wait)) return;
     PlocRound g{a.cluster[0], a.cluster[1], a.n, a.n - 2, 1, false, 0};
     while (g.nc > kPlocSolo) {
         // the most lanes a cluster with which every block still has one tile at most
@@ -854,7 +861,7 @@ __global__ void __launch_bounds__(kPlocThreads, 1) k_ploc(PlocArgs a)
             g.C = g.D;
             g.D = const_cast<float4*>(swap);
         }
-        if (!build_meet(a.place, blocks, met, a.status)) return;
+        if (!build_meet(a.place, blocks, met, a.wait)) return;
     }
     if (blockIdx.x == 0) ploc_solo(a, g.C, g.nc, g.id_top, s_c, s_nn);
 }
@@ -877,7 +884,8 @@ size_t ploc_scratch_bytes(int64_t n)
 }
 
 cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, float4* nodes_out, int* max_height_dev,
-                       int radius, void* scratch, size_t scratch_bytes, AreaW w, int* status, int num_sms, int coop)
+                       int radius, void* scratch, size_t scratch_bytes, AreaW w, int* status, int num_sms, int coop,
+                       uint64_t wait_ns)
 {
     if (n < 2 || radius < 1 || radius > kPlocMaxRadius) return cudaErrorInvalidValue;
     if (scratch_bytes < ploc_scratch_bytes(n)) return cudaErrorInvalidValue;
@@ -898,7 +906,7 @@ cudaError_t build_ploc(cudaStream_t s, const float4* tris_sorted, int64_t n, flo
     a.max_height = max_height_dev;
     a.radius = radius;
     a.w = w;
-    a.status = status;
+    a.wait = BuildWait{status, wait_ns};
     cudaError_t e = cudaMemsetAsync(zero, 0, (size_t)(p - zero), s);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_ploc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlocShared);
@@ -1202,7 +1210,7 @@ struct CollapseArgs {
     const float4* bn;
     int use_dp;
     CollapseTree tree[2];  // 4-wide, 8-wide
-    int* status;
+    BuildWait wait;
 };
 
 template <int W>
@@ -1242,7 +1250,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
         // internal children of the tiles before this block's, and of all
         unsigned at = 0, next = sum;
         if (shared) {
-            if (!build_meet(c.place, of, met, a.status)) return false;
+            if (!build_meet(c.place, of, met, a.wait)) return false;
             unsigned mine = 0, all = 0;
             for (int t = tid; t < tiles; t += T) {
                 const unsigned v = __ldcg(&c.total[t]);
@@ -1286,7 +1294,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
         base += n;
         n = (int)next;
         ++levels;
-        return build_meet(c.place, of, met, a.status);
+        return build_meet(c.place, of, met, a.wait);
     };
     // the first levels fit one block, which walks them alone while the others wait once
     if (blocks > 1) {
@@ -1298,7 +1306,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
                 __stcg(&c.state[2], levels);
             }
         }
-        if (!build_meet(c.place, blocks, met, a.status)) return;
+        if (!build_meet(c.place, blocks, met, a.wait)) return;
         n = __ldcg(&c.state[0]);
         base = __ldcg(&c.state[1]);
         levels = __ldcg(&c.state[2]);
@@ -1323,7 +1331,7 @@ __device__ void collapse_levels(const CollapseArgs& a, const CollapseTree& c, un
 __global__ void __launch_bounds__(kCollapseThreads) k_collapse_levels(const __grid_constant__ CollapseArgs a)
 {
     // a build that failed left no tree to walk
-    if (*(volatile int*)a.status != ST_OK) return;
+    if (*(volatile int*)a.wait.status != ST_OK) return;
     if ((blockIdx.x & 1u) == 0) collapse_levels<4>(a, a.tree[0], blockIdx.x >> 1, gridDim.x >> 1);
     else collapse_levels<8>(a, a.tree[1], blockIdx.x >> 1, gridDim.x >> 1);
 }
@@ -1427,7 +1435,7 @@ size_t collapse_scratch_bytes(int64_t n_binary, int sah_dp)
 // are (4-wide, 8-wide).
 cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_binary, void* scratch,
                           size_t scratch_bytes, int sah_dp, float tri_cost, AreaW area_w, int* status, int num_sms,
-                          int coop, WideInfo info_dev[2])
+                          int coop, uint64_t wait_ns, WideInfo info_dev[2])
 {
     if (n_binary < 1) return cudaErrorInvalidValue;
     if (n_binary < 2) sah_dp = 0;  // a single triangle: nothing to choose
@@ -1435,7 +1443,7 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
     if (scratch_bytes < c.bytes) return cudaErrorInvalidValue;
     c.a.bn = binary_nodes;
     c.a.use_dp = sah_dp ? 1 : 0;
-    c.a.status = status;
+    c.a.wait = BuildWait{status, wait_ns};
     for (CollapseTree& t : c.a.tree) {
         t.dp.w = area_w;  // the largest-area rule reads it too
         t.dp.c_node = 1.0f;

@@ -157,8 +157,8 @@ struct BuildScratch;
 cudaError_t build_lbvh(cudaStream_t s, const float* verts, int64_t n_verts, const uint32_t* tris,
                        const uint16_t* mat, const uint32_t* inst, int64_t n_tris, float4* nodes_out,
                        float4* tris_out, uint32_t* leaf_tri_out, int* status, int* max_depth_dev,
-                       void* scratch, size_t scratch_bytes, int num_sms, int coop, int method = 0,
-                       int ploc_radius = 16, AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
+                       void* scratch, size_t scratch_bytes, int num_sms, int coop, uint64_t wait_ns,
+                       int method = 0, int ploc_radius = 16, AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});
 // scratch of the clustering build (method 1), on top of nothing: it reuses build_lbvh's scratch
 size_t ploc_scratch_bytes(int64_t n_tris);
 size_t build_scratch_bytes(int64_t n_tris);
@@ -179,7 +179,7 @@ struct BuildResult {
 };
 cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_binary, void* scratch,
                           size_t scratch_bytes, int sah_dp, float tri_cost, AreaW area_w, int* status, int num_sms,
-                          int coop, WideInfo info_dev[2]);
+                          int coop, uint64_t wait_ns, WideInfo info_dev[2]);
 cudaError_t collapse_write(cudaStream_t s, int width, const float4* binary_nodes, int64_t n_binary, float4* nodes,
                            int64_t n_wide, void* scratch, int sah_dp, AreaW area_w);
 size_t collapse_scratch_bytes(int64_t n_binary, int sah_dp);

@@ -433,14 +433,15 @@ lidar_status lidar_scene_build(lidar_ctx* c, const float* verts, int64_t n_verts
         cudaEventRecord(e0, c->stream);
         cudaError_t e = build_lbvh(c->stream, verts, n_verts, tris, mat, inst, n_tris, s->nodes, s->tris,
                                    s->leaf_tri, c->status_dev, &c->build_dev->height, c->scratch, c->scratch_bytes,
-                                   c->num_sms, c->coop, n_tris >= 2 ? c->build_method : 0, c->ploc_radius, c->area_w);
+                                   c->num_sms, c->coop, c->cfg.wait_ns, n_tris >= 2 ? c->build_method : 0,
+                                   c->ploc_radius, c->area_w);
         if (e == cudaSuccess && c->treelet_rounds > 0)
             e = restructure_treelets(c->stream, s->tris, n_tris, s->nodes, &c->build_dev->height, c->treelet_rounds,
                                      c->tri_cost, c->scratch, c->scratch_bytes, &c->build_dev->treelets, c->status_dev,
                                      c->area_w);
         if (e == cudaSuccess)
             e = collapse_plan(c->stream, s->nodes, s->n_nodes, c->scratch, c->scratch_bytes, c->collapse, c->tri_cost,
-                              c->area_w, c->status_dev, c->num_sms, c->coop, c->build_dev->wide);
+                              c->area_w, c->status_dev, c->num_sms, c->coop, c->cfg.wait_ns, c->build_dev->wide);
         cudaEventRecord(e1, c->stream);
         if (e != cudaSuccess) {
             set_error(std::string("lidar_scene_build: ") + cudaGetErrorString(e));
