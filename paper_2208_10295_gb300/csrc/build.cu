@@ -1016,21 +1016,29 @@ __global__ void k_parents(const float4* __restrict__ bn, int n_binary, int* pare
 
 // one thread per triangle climbs towards the root; the second child to finish
 // computes its parent's table, so every node is computed once, after both
-// children
+// children.  A clustering that gave up leaves no tree (its status is set by
+// then) but unwritten links: nothing is read then.
 template <int W>
-__global__ void k_collapse_dp(const float4* __restrict__ bn, int n_leaves, CollapseDP dp)
+__global__ void k_collapse_dp(const float4* __restrict__ bn, int n_leaves, CollapseDP dp, int* status)
 {
+    if (*(volatile int*)status != ST_OK) return;
     const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
     if (leaf >= n_leaves) return;
     int node = dp.parent_leaf[leaf];
     while (node >= 0) {
         __threadfence();
-        if (atomicAdd(&dp.visits[node], 1u) == 0u) return;  // the other child is still running
+        // only the second arrival goes on (the other child is still running at
+        // the first; links in a circle would bring more), so every climb ends
+        if (atomicAdd(&dp.visits[node], 1u) != 1u) return;
         __threadfence();
         ChildBox cb[2];
         float cc[2][W];
         for (int side = 0; side < 2; ++side) {
             binary_child(bn, node, side, cb[side]);
+            if (cb[side].ref >= n_leaves - 1) {
+                raise_status(status, ST_BOUNDS);
+                return;
+            }
             if (cb[side].ref < 0) {
                 const float v = dp.c_tri * half_area(cb[side], dp.w);
                 for (int i = 0; i < W; ++i) cc[side][i] = v;
@@ -1456,15 +1464,17 @@ cudaError_t collapse_plan(cudaStream_t s, const float4* binary_nodes, int64_t n_
     if (e != cudaSuccess) return e;
     if (sah_dp) {
         const int nb = (int)n_binary;
+        // no parent (-1) but where k_parents finds a link
         e = cudaMemsetAsync(c.parent_node, 0xFF, (size_t)nb * sizeof(int), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c.parent_leaf, 0xFF, ((size_t)nb + 1) * sizeof(int), s);
         if (e != cudaSuccess) return e;
         k_parents<<<(nb + 255) / 256, 256, 0, s>>>(binary_nodes, nb, c.parent_node, c.parent_leaf, nullptr);
         for (int k = 0; k < 2; ++k) {
             const CollapseDP& dp = c.a.tree[k].dp;
             e = cudaMemsetAsync(dp.visits, 0, (size_t)nb * sizeof(unsigned), s);
             if (e != cudaSuccess) return e;
-            if (k == 0) k_collapse_dp<4><<<(nb + 1 + 255) / 256, 256, 0, s>>>(binary_nodes, nb + 1, dp);
-            else k_collapse_dp<8><<<(nb + 1 + 255) / 256, 256, 0, s>>>(binary_nodes, nb + 1, dp);
+            if (k == 0) k_collapse_dp<4><<<(nb + 1 + 255) / 256, 256, 0, s>>>(binary_nodes, nb + 1, dp, status);
+            else k_collapse_dp<8><<<(nb + 1 + 255) / 256, 256, 0, s>>>(binary_nodes, nb + 1, dp, status);
         }
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

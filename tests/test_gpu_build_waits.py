@@ -58,9 +58,17 @@ def test_clustering_gives_up(L, n, treelet_rounds):
     _times_out_and_recovers(L, n, method=1, collapse=0, treelet_rounds=treelet_rounds)
 
 
+@pytest.mark.parametrize("n", [5000, 70001])
+@pytest.mark.parametrize("treelet_rounds", [0, 3])
+def test_clustering_gives_up_before_the_dynamic_program(L, n, treelet_rounds):
+    """The collapse's program climbs the tree that the clustering did not finish: it must read none of it."""
+    _times_out_and_recovers(L, n, method=1, collapse=1, treelet_rounds=treelet_rounds)
+
+
 def test_collapse_gives_up(L):
     """The tree is whole (the Karras build has no such waits): the levels of the wide trees give up."""
-    _times_out_and_recovers(L, 70001, method=0, collapse=0, treelet_rounds=0)
+    for collapse in (0, 1):
+        _times_out_and_recovers(L, 70001, method=0, collapse=collapse, treelet_rounds=0)
 
 
 def test_one_block_waits_for_nobody(L):
