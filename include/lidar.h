@@ -98,6 +98,11 @@ lidar_status lidar_scene_build(lidar_ctx* ctx, const float* verts_dev, int64_t n
                                const uint16_t* tri_material_dev, const uint32_t* tri_instance_dev,
                                lidar_scene** out);
 
+/* Frees a scene once the device has finished all work launched on it, on any
+ * stream (a replayed graph's as well as the context's).  Up to 1 GiB of the
+ * memory of freed scenes stays with the context for the next ones (a rebuild
+ * then maps none); lidar_destroy gives it back, what is above that goes back
+ * when the context's stream is next synchronised. */
 void lidar_scene_free(lidar_scene* scene);
 
 typedef struct {

@@ -333,7 +333,10 @@ void lidar_scene_free(lidar_scene* s)
 {
     if (!s) return;
     DeviceGuard g(s->ctx->device);
-    cudaStreamSynchronize(s->ctx->stream);
+    // The pool orders the arrays' next use after this context's stream only; a
+    // caller's graph may be reading them on another one, for which cudaFree
+    // would have waited.
+    cudaDeviceSynchronize();
     scene_release(s->ctx, s->nodes);
     scene_release(s->ctx, s->nodes4);
     scene_release(s->ctx, s->nodes8);
