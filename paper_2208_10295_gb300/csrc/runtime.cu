@@ -217,17 +217,18 @@ cudaMemPool_t create_pool(int device)
 
 cudaError_t scene_alloc(lidar_ctx* c, void** p, size_t bytes)
 {
+    *p = nullptr;
+    // a build synchronises, which a capture cannot hold: refused here, as
+    // cudaMalloc would refuse it, and not turned into a node of the graph (nor
+    // is the pool asked for, which a capture refuses for good)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+        return cudaErrorStreamCaptureUnsupported;
     if (!c->pool_tried) {
         c->pool = create_pool(c->device);
         c->pool_tried = true;
     }
     if (!c->pool) return dev_alloc(p, bytes);
-    *p = nullptr;
-    // a build synchronises, which a capture cannot hold: refused here, as
-    // cudaMalloc would refuse it, and not turned into a node of the graph
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
-        return cudaErrorStreamCaptureUnsupported;
     if (alloc_fault()) return cudaErrorMemoryAllocation;
     return cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
 }
