@@ -553,8 +553,8 @@ lidar_status lidar_raster_gbuffer(lidar_ctx* ctx, const lidar_scene* scene, cons
 /* --------------------------------------------------------------- launch tuning */
 
 typedef struct {
-    int32_t block_threads;   /* threads per block of the cast kernel (multiple of 32, <= 256) */
-    int32_t blocks_per_sm;   /* persistent blocks per SM */
+    int32_t block_threads;   /* threads per block of the cast kernel (multiple of 32, <= 256), or 0 */
+    int32_t blocks_per_sm;   /* persistent blocks per SM, or 0 */
     int32_t tile_rays;       /* rays a warp takes from the work counter at a time (multiple of 32) */
     int32_t ray_order;       /* 0 = beam order, 1 = Morton order of beam directions */
     int32_t traversal;       /* binary tree: 0 = each lane tests its triangles as it meets them,
@@ -566,10 +566,12 @@ typedef struct {
                                 wait (cooperative launch); 0: as a separate kernel */
 } lidar_launch_config;
 
-/* The default is 128 threads x 4 blocks.  Until a call sets block_threads or
- * blocks_per_sm to another value, casts and sweeps with traversal 2 choose how
- * many threads to keep resident by the number of rays (512 a SM for few, up to
- * 1,024 for many); afterwards they run as set, the default values included. */
+/* block_threads and blocks_per_sm both 0 (the default, and what the getter
+ * returns then) leave the shape to the library: casts and sweeps with traversal
+ * 2 choose how many threads to keep resident by the number of rays (512 a SM
+ * for few, up to 1,024 for many), the other traversals run 128 threads x 4
+ * blocks.  With either set, all run as set, a 0 beside it standing for 128 or
+ * 4. */
 lidar_status lidar_get_launch_config(lidar_ctx* ctx, lidar_launch_config* out);
 lidar_status lidar_set_launch_config(lidar_ctx* ctx, const lidar_launch_config* cfg);
 

@@ -112,6 +112,9 @@ static SceneDev scene_dev(const lidar_scene* scene)
                     scene->nodes4, scene->n_nodes4, scene->nodes8, scene->n_nodes8};
 }
 
+// the launch shape where the library chooses none by the work, and of a field a caller leaves at 0
+constexpr int kDefaultThreads = 128, kDefaultBlocks = 4;
+
 struct lidar_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -145,8 +148,8 @@ struct lidar_ctx {
     int overlap = 1;         // consecutive direct casts may overlap (programmatic dependent launch)
     int dense_cur = 0;       // which half of the scratch the next direct cast's dense records use
     std::vector<std::pair<uintptr_t, uintptr_t>> last_out;  // output byte ranges of the last direct cast
-    LaunchCfg cfg{128, 4, 32, 1, 2, 1};
-    bool own_shape = true;    // nobody has set another block_threads or blocks_per_sm: see launch_shape
+    LaunchCfg cfg{kDefaultThreads, kDefaultBlocks, 32, 1, 2, 1};
+    bool own_shape = true;    // no caller has set block_threads or blocks_per_sm: see launch_shape
     int build_method = 1;     // 0 Karras LBVH, 1 PLOC clustering (fewer node fetches per ray)
     int ploc_radius = 16;
     int collapse = 0;         // wide nodes: 0 open the largest child, 1 SAH dynamic program
@@ -704,8 +707,8 @@ lidar_status lidar_set_materials(lidar_ctx* c, const float* table, int32_t M)
 }
 
 // Launch configuration of a cast or sweep of `ray_tiles` (32 rays each).  As
-// long as no caller has set block_threads or blocks_per_sm to anything but the
-// default, the library chooses how many threads stay resident: few tiles end
+// long as no caller has set block_threads or blocks_per_sm, the library chooses
+// how many threads stay resident: few tiles end
 // with their longest walks, which want the fewest neighbours (512 threads a
 // SM); many are bound by issue and want the most warps (1,024 at 64
 // registers).  Measured with the 4-wide walk, us, 512 / 768 / 1,024 threads a
@@ -1729,8 +1732,8 @@ lidar_status lidar_get_build_options(lidar_ctx* c, lidar_build_options* o)
 lidar_status lidar_get_launch_config(lidar_ctx* c, lidar_launch_config* out)
 {
     LIDAR_CHECK_ARG(c != nullptr && out != nullptr, "lidar_get_launch_config: NULL argument");
-    out->block_threads = c->cfg.block_threads;
-    out->blocks_per_sm = c->cfg.blocks_per_sm;
+    out->block_threads = c->own_shape ? 0 : c->cfg.block_threads;
+    out->blocks_per_sm = c->own_shape ? 0 : c->cfg.blocks_per_sm;
     out->tile_rays = c->cfg.tile_rays;
     out->ray_order = c->cfg.ray_order;
     out->traversal = c->cfg.traversal;
@@ -1741,9 +1744,10 @@ lidar_status lidar_get_launch_config(lidar_ctx* c, lidar_launch_config* out)
 lidar_status lidar_set_launch_config(lidar_ctx* c, const lidar_launch_config* cfg)
 {
     LIDAR_CHECK_ARG(c != nullptr && cfg != nullptr, "lidar_set_launch_config: NULL argument");
-    LIDAR_CHECK_ARG(cfg->block_threads >= 32 && cfg->block_threads <= 256 && cfg->block_threads % 32 == 0,
-                    "lidar_set_launch_config: block_threads must be a multiple of 32 in [32, 256]");
-    LIDAR_CHECK_ARG(cfg->blocks_per_sm >= 1 && cfg->blocks_per_sm <= 64, "lidar_set_launch_config: blocks_per_sm in [1, 64]");
+    LIDAR_CHECK_ARG(cfg->block_threads >= 0 && cfg->block_threads <= 256 && cfg->block_threads % 32 == 0,
+                    "lidar_set_launch_config: block_threads must be 0 or a multiple of 32 in [32, 256]");
+    LIDAR_CHECK_ARG(cfg->blocks_per_sm >= 0 && cfg->blocks_per_sm <= 64,
+                    "lidar_set_launch_config: blocks_per_sm must be 0 or in [1, 64]");
     LIDAR_CHECK_ARG(cfg->tile_rays >= 32 && cfg->tile_rays <= (1 << 20) && cfg->tile_rays % 32 == 0,
                     "lidar_set_launch_config: tile_rays must be a multiple of 32 in [32, 2^20]");
     LIDAR_CHECK_ARG(cfg->ray_order == 0 || cfg->ray_order == 1, "lidar_set_launch_config: ray_order is 0 or 1");
@@ -1751,9 +1755,9 @@ lidar_status lidar_set_launch_config(lidar_ctx* c, const lidar_launch_config* cf
     LIDAR_CHECK_ARG(cfg->fused_scatter == 0 || cfg->fused_scatter == 1,
                     "lidar_set_launch_config: fused_scatter is 0 or 1");
     DeviceGuard g(c->device);
-    if (cfg->block_threads != c->cfg.block_threads || cfg->blocks_per_sm != c->cfg.blocks_per_sm) c->own_shape = false;
-    c->cfg.block_threads = cfg->block_threads;
-    c->cfg.blocks_per_sm = cfg->blocks_per_sm;
+    c->own_shape = cfg->block_threads == 0 && cfg->blocks_per_sm == 0;
+    c->cfg.block_threads = cfg->block_threads ? cfg->block_threads : kDefaultThreads;
+    c->cfg.blocks_per_sm = cfg->blocks_per_sm ? cfg->blocks_per_sm : kDefaultBlocks;
     c->cfg.tile_rays = cfg->tile_rays;
     c->cfg.ray_order = cfg->ray_order;
     c->cfg.traversal = cfg->traversal;

@@ -365,11 +365,14 @@ class Lidar:
 
     # ----------------------------------------------------------- tuning
     def launch_config(self):
+        """The launch configuration; block_threads and blocks_per_sm are 0 while the library chooses them."""
         c = C.lidar_launch_config()
         C.check(C.lidar_get_launch_config(self.handle, ctypes.byref(c)), "lidar_get_launch_config")
         return {k: getattr(c, k) for k, _ in c._fields_}
 
     def set_launch_config(self, **kw):
+        """Fields not given keep their current values; block_threads=0, blocks_per_sm=0 hands the launch shape back to
+        the library."""
         cur = self.launch_config()
         cur.update(kw)
         c = C.lidar_launch_config(**cur)

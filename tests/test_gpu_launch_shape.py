@@ -1,6 +1,7 @@
 """The launch shape and the order of the work change no result: what the library chooses by the number of rays against
 shapes that a caller sets, and frames and sweeps of equal size, whose tiles take turns, against ones cast beside a
 frame of another size, which do not."""
+import ctypes
 import dataclasses
 
 import numpy as np
@@ -91,3 +92,77 @@ def test_turns_of_equal_frames(make, n_frames, beams_off, n_subrays, sweep):
     mixed = np.concatenate([turns, turns[:1]])
     mixed[-1]["sensor"] = 1
     _same(_cast(lid, scene, w, turns, sweep), _cast(lid, scene, w, mixed, sweep), lid.total_beams(turns))
+
+
+class _KernelParams(ctypes.Structure):
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("shared", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kernel", ctypes.c_void_p), ("context", ctypes.c_void_p)]
+
+
+def _captured_shape(lid, batch, scene, w, beams):
+    """Threads per block and blocks per SM of the kernel that a cast of the batch launches, from a stream capture."""
+    cuda = ctypes.CDLL("libcuda.so.1")
+    stream, graph, n = ctypes.c_void_p(lid.stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert cuda.cuStreamBeginCapture_v2(stream, 2) == 0  # relaxed
+    try:
+        batch.cast_into(scene, w.seed, beams)
+    finally:
+        assert cuda.cuStreamEndCapture(stream, ctypes.byref(graph)) == 0
+    assert cuda.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cuda.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    shapes = []
+    for node in nodes:
+        kind, p = ctypes.c_int(), _KernelParams()
+        assert cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:  # a kernel
+            assert cuda.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+            shapes.append((p.block[0], p.grid[0] / torch.cuda.get_device_properties(0).multi_processor_count))
+    cuda.cuGraphDestroy(graph)
+    assert len(shapes) == 1  # a dense cast is one kernel
+    return shapes[0]
+
+
+def test_whose_shape_a_cast_runs(make):
+    """A shape that a caller sets is what runs, the default values from the first call on included; other fields leave
+    it alone; two zeros hand it back."""
+    from paper_2208_10295_gb300 import Lidar, capi
+    lid = Lidar(0, torch.cuda.Stream())
+    try:
+        w = _workload(3, 1024, 3, 7)  # more tiles than any shape below keeps resident
+        scene = setup(lid, w)[0]
+        frames = w.frames[:3]
+        beams = lid.alloc_beams(lid.total_beams(frames), ("valid",))
+        batch = lid.batch(frames)
+        batch.cast_into(scene, w.seed, beams)
+        assert lid.sync_status() == 0
+
+        def now():
+            c = lid.launch_config()
+            return (c["block_threads"], c["blocks_per_sm"]), _captured_shape(lid, batch, scene, w, beams)
+        own = now()
+        assert own[0] == (0, 0) and own[1][0] == 256
+        lid.set_launch_config(ray_order=0)
+        assert now() == own
+        lid.set_launch_config(ray_order=1, block_threads=128, blocks_per_sm=4)
+        assert now() == ((128, 4), (128, 4))
+        lid.set_launch_config(ray_order=1)
+        assert now() == ((128, 4), (128, 4))
+        kept = lid.launch_config()
+        lid.set_launch_config(block_threads=64, blocks_per_sm=0)
+        assert now() == ((64, 4), (64, 4))
+        lid.set_launch_config(block_threads=0, blocks_per_sm=2)
+        assert now() == ((128, 2), (128, 2))
+        lid.set_launch_config(**kept)
+        assert now() == ((128, 4), (128, 4))
+        lid.set_launch_config(block_threads=0, blocks_per_sm=0)
+        assert now() == own
+        for bad in ({"block_threads": -32}, {"blocks_per_sm": -1}, {"block_threads": 288}, {"blocks_per_sm": 65}):
+            with pytest.raises(capi.LidarError) as e:
+                lid.set_launch_config(**bad)
+            assert e.value.status == capi.LIDAR_EINVAL
+        assert now() == own
+        batch.free()
+    finally:
+        lid.close()
