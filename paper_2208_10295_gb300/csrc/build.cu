@@ -1556,11 +1556,15 @@ struct TreeletArgs {
     unsigned* expect;         // [n_binary] children the round visits
     unsigned* visits;         // [n_binary] of these, finished; zero at the start of a round
     float* cost;              // [n_binary] surface-area cost of each node's subtree
-    // A treelet is a function of its subtree alone (the costs of its leaves
-    // among it, to the last bit), so one that was kept and whose subtree is as
-    // it was is kept again without a look: mark[n] is the last round (1, 2,
-    // ...) that rewrote node n, up[n] the last one that changed a node or a
-    // cost of n's subtree before it was done with n.
+    // A treelet is a function of the nodes it opens and the costs of its leaves,
+    // all at most kTreeletReach levels below its root, so one that was kept and
+    // below which no node was rewritten and no cost moved (in its last bit) that
+    // near is kept again without a look: mark[n] is the last round (1, 2, ...)
+    // that rewrote node n; up[n] has, in its low four bits, the last round that
+    // changed a node or a cost in n's subtree near enough for n's parent, and
+    // above them how many levels below n (0: n itself) the nearest is.  (A change
+    // a few levels down need not move the costs above it: they may be so much
+    // larger that it is lost in their rounding.)
     uint8_t* mark;            // [n_binary]
     uint8_t* up;              // [n_binary]
     int round;
@@ -1569,6 +1573,9 @@ struct TreeletArgs {
     float c_node, c_tri;
     AreaW w;                  // face weights of the area measure
 };
+
+// a chain of kTreeletLeaves - 1 internal nodes, the root the first, has its last leaves this far below
+constexpr int kTreeletReach = kTreeletLeaves - 1;
 
 // longest climb a valid hierarchy of up to 2^31 triangles can need is far
 // below this; a longer one means a broken tree (a cycle), which ends the climb
@@ -1973,7 +1980,9 @@ __global__ void __launch_bounds__(kBuildThreads) k_treelet_paths(TreeletArgs a)
 // with the treelets whose subtree is unchanged kept unseen 1.2, 0.88, 0.64,
 // 0.51, 0.41, 0.35, 0.31, 0.30 ms; climbing only where something was rewritten
 // and with one acquire-release arrival a level 1.14, 0.83, 0.60, 0.42, 0.32,
-// 0.30, 0.25, 0.24 ms.  A stride between a warp's nodes, fewer lanes or more
+// 0.30, 0.25, 0.24 ms.  (Looking kTreeletReach levels above every change, and
+// not only while it still moves the costs, took the whole load from 5.21 to
+// 5.31 ms; it is what makes the rounds those of a full evaluation.)  A stride between a warp's nodes, fewer lanes or more
 // nodes a warp all took longer: neighbours share the climb.
 __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_round(TreeletArgs a)
 {
@@ -1990,7 +1999,8 @@ __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_rou
         }
         int2 c = make_int2(-1, -1);
         int parent = -1;
-        bool look = false, below = false;  // the warp has to look at the treelet; its subtree changed this round
+        bool look = false;           // the warp has to look at the treelet
+        int levels = kTreeletReach;  // below the node is the nearest change of this round (or more)
         if (node >= 0) {
             const unsigned before = step > 0 ? arrive(&a.visits[node]) + 1u : 0u;
             const unsigned expect = a.expect[node];
@@ -2016,24 +2026,27 @@ __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_rou
                 const float cost = subtree_cost(a, c.x, L), other = subtree_cost(a, c.y, R);
                 tbox_grow(L, R);
                 const float now = a.c_node * tbox_area(L, a.w) + cost + other;
-                below = __float_as_int(__ldcg(&a.cost[node])) != __float_as_int(now);
+                if (__float_as_int(__ldcg(&a.cost[node])) != __float_as_int(now)) levels = 0;
                 a.cost[node] = now;
                 look = false;
             }
         } else {
-            below = (c.x >= 0 && __ldcg(&a.up[c.x]) == a.round) || (c.y >= 0 && __ldcg(&a.up[c.y]) == a.round);
-            look = look || below;
-            below = false;
+            auto nearest = [&](int child) {
+                const int up = child >= 0 ? __ldcg(&a.up[child]) : 0;
+                return (up & 15) == a.round ? (up >> 4) + 1 : kTreeletReach + 1;
+            };
+            levels = min(nearest(c.x), nearest(c.y));
+            look = look || levels <= kTreeletReach;
         }
         for (unsigned todo = __ballot_sync(0xffffffffu, look); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
             const int did = treelet_node(a, __shfl_sync(0xffffffffu, node, src), t, sub2, sub3a, sub3b);
             if (lane == src) {
                 if (did < 0) raise_status(a.status, ST_BOUNDS);
-                below = did > 0;
+                if (did > 0) levels = 0;
             }
         }
-        if (below) a.up[node] = (uint8_t)a.round;
+        if (node >= 0 && levels < kTreeletReach) a.up[node] = (uint8_t)(levels << 4 | a.round);
         __syncwarp();  // every lane's writes, before a lane's arrival releases them
         node = node >= 0 ? parent : -1;
     }
