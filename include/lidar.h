@@ -463,6 +463,10 @@ lidar_status lidar_schedule_by_cost(lidar_ctx* ctx, const lidar_scene* scene, co
 /* Restores the default order of a slot. */
 lidar_status lidar_reset_schedule(lidar_ctx* ctx, int32_t slot);
 
+/* Gives a slot the plain Morton order of its beam directions, for sensors whose
+ * level beams do not take the longest (looking down, rolled). */
+lidar_status lidar_morton_schedule(lidar_ctx* ctx, int32_t slot);
+
 /* --------------------------------------------- rolling shutter, multi-echo */
 
 /* One sweep of a spinning sensor: the sensor-to-world pose at its start and
@@ -556,7 +560,7 @@ typedef struct {
     int32_t block_threads;   /* threads per block of the cast kernel (multiple of 32, <= 256), or 0 */
     int32_t blocks_per_sm;   /* persistent blocks per SM, or 0 */
     int32_t tile_rays;       /* rays a warp takes from the work counter at a time (multiple of 32) */
-    int32_t ray_order;       /* 0 = beam order, 1 = Morton order of beam directions */
+    int32_t ray_order;       /* 0 = beam order, 1 = the slot's ray schedule (lidar_schedule_by_cost) */
     int32_t traversal;       /* binary tree: 0 = each lane tests its triangles as it meets them,
                                 1 = warp-synchronous with postponed triangle tests;
                                 2 = 4-wide tree, per lane, children visited near to far;

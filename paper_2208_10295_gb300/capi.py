@@ -148,6 +148,7 @@ _PROTOS = [
     ("lidar_schedule_by_cost", ctypes.c_int, [c_vp, c_vp, ctypes.POINTER(lidar_frame), ctypes.c_uint64,
                                               ctypes.c_int32]),
     ("lidar_reset_schedule", ctypes.c_int, [c_vp, ctypes.c_int32]),
+    ("lidar_morton_schedule", ctypes.c_int, [c_vp, ctypes.c_int32]),
     ("lidar_cast_sweep", ctypes.c_int, [c_vp, c_vp, c_vp, ctypes.c_int32, ctypes.c_uint64,
                                         ctypes.POINTER(lidar_beams), ctypes.POINTER(lidar_echoes)]),
     ("lidar_raster_cast", ctypes.c_int, [c_vp, c_vp, c_vp, ctypes.c_int32, ctypes.c_uint64,
@@ -239,6 +240,7 @@ lidar_get_build_options = _fwd("lidar_get_build_options")
 lidar_raster_gbuffer = _fwd("lidar_raster_gbuffer")
 lidar_schedule_by_cost = _fwd("lidar_schedule_by_cost")
 lidar_reset_schedule = _fwd("lidar_reset_schedule")
+lidar_morton_schedule = _fwd("lidar_morton_schedule")
 lidar_get_launch_config = _fwd("lidar_get_launch_config")
 lidar_set_launch_config = _fwd("lidar_set_launch_config")
 lidar_set_wait_limit = _fwd("lidar_set_wait_limit")

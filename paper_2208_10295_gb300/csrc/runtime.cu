@@ -1694,6 +1694,22 @@ lidar_status lidar_reset_schedule(lidar_ctx* c, int32_t slot)
     return LIDAR_OK;
 }
 
+lidar_status lidar_morton_schedule(lidar_ctx* c, int32_t slot)
+{
+    LIDAR_CHECK_ARG(c != nullptr, "lidar_morton_schedule: ctx is NULL");
+    LIDAR_CHECK_ARG(slot >= 0 && slot < LIDAR_MAX_SENSORS, "lidar_morton_schedule: slot out of range");
+    if (!c->slots[slot].set) {
+        set_error("lidar_morton_schedule: no sensor in this slot");
+        return LIDAR_ESTATE;
+    }
+    DeviceGuard g(c->device);
+    SensorSlot& sl = c->slots[slot];
+    LIDAR_CUDA(cudaMemcpyAsync(sl.order_dev, sl.base_order_dev, sl.n_beams * sizeof(uint32_t),
+                               cudaMemcpyDeviceToDevice, c->stream));
+    LIDAR_CUDA(cudaStreamSynchronize(c->stream));
+    return LIDAR_OK;
+}
+
 lidar_status lidar_set_build_options(lidar_ctx* c, const lidar_build_options* o)
 {
     LIDAR_CHECK_ARG(c != nullptr && o != nullptr, "lidar_set_build_options: NULL argument");

@@ -290,7 +290,12 @@ class Lidar:
                                          ctypes.c_uint64(seed), int(mode)), "lidar_schedule_by_cost")
 
     def reset_schedule(self, slot: int):
+        """The default ray order: 32-beam groups of the Morton order, most level first."""
         C.check(C.lidar_reset_schedule(self.handle, slot), "lidar_reset_schedule")
+
+    def morton_schedule(self, slot: int):
+        """The plain Morton order of the slot's beam directions."""
+        C.check(C.lidar_morton_schedule(self.handle, slot), "lidar_morton_schedule")
 
     # ----------------------------------------------------------- sweeps and echoes
     def alloc_echoes(self, n: int, n_echoes: int):

@@ -2,9 +2,10 @@
 
 Searches threads per block x resident blocks per SM (which also picks the
 register budget: up to 512 threads per SM 128 registers, up to 768 85, more
-64), the traversal variant, the ray order (beam order / Morton
-order of directions), the schedule (Morton groups / most expensive groups
-first / per-beam cost buckets) and, when the point cloud is timed too, whether
+64), the traversal variant, the ray order (beam order / the schedule's), the
+schedule (Morton order of directions / its groups most level first, the
+default / its groups most expensive first / per-beam cost buckets) and, when
+the point cloud is timed too, whether
 the ordered scatter runs inside the cast (cooperative launch) or as its own
 kernel, timing each candidate with CUDA events on the context stream.  Every
 candidate produces bit-identical results (tested), so the choice is purely a
@@ -29,7 +30,7 @@ SPACE = {
     "blocks_per_sm": (2, 3, 4, 6, 8, 12),
     "traversal": (0, 1, 2, 3),
     "ray_order": (0, 1),
-    "schedule": ("morton", "cost", "bucket"),
+    "schedule": ("morton", "level", "cost", "bucket"),
     "fused_scatter": (0, 1),
 }
 
@@ -92,7 +93,7 @@ def candidates(points=False, wide8=True, restrict=None):
         if tv == 3 and not wide8:
             continue  # the scene kept no 8-wide tree
         if ro == 0 and sc != "morton":
-            continue  # the cost schedules reorder the Morton order
+            continue  # beam order knows no schedule (named by the first)
         if not points and fs == 0:
             continue  # without a point cloud there is no scatter
         yield {"block_threads": bt, "blocks_per_sm": bps, "tile_rays": 32, "traversal": tv, "ray_order": ro,
@@ -103,7 +104,10 @@ def apply(L, scene, cfg, schedule_frames, seed):
     L.set_launch_config(**{k: v for k, v in cfg.items() if k != "schedule"})
     slots = sorted({int(s) for s in np.ascontiguousarray(schedule_frames)["sensor"]})
     for s in slots:
-        L.reset_schedule(s)
+        if cfg.get("schedule") == "morton":
+            L.morton_schedule(s)
+        else:
+            L.reset_schedule(s)
     if cfg.get("schedule") in ("cost", "bucket"):
         fr = np.ascontiguousarray(schedule_frames)
         for s in slots:
