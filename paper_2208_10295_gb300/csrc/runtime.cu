@@ -706,32 +706,44 @@ lidar_status lidar_set_materials(lidar_ctx* c, const float* table, int32_t M)
     return LIDAR_OK;
 }
 
-// Launch configuration of a cast or sweep of `ray_tiles` (32 rays each).  As
-// long as no caller has set block_threads or blocks_per_sm, the library chooses
-// how many threads stay resident: few tiles end
-// with their longest walks, which want the fewest neighbours (512 threads a
-// SM); many are bound by issue and want the most warps (1,024 at 64
-// registers).  Measured with the 4-wide walk, us, 512 / 768 / 1,024 threads a
-// SM: 8,192 tiles (a 128 x 2048 frame in 1M triangles) 108 / 107 / 116, 16,384
-// 158 / 152 / 158, 32,768 286 / 251 / 253, 65,536 571 / 484 / 453; a city's
-// 57,344 (seven sub-rays) 421 / 386 / 426, 114,688 773 / 682 / 667; a rig's
-// 31,000 294 / 269 / 267, 123,000 1024 / 876 / 833.  256-thread blocks took 1-8
-// % less than 128-thread ones at each.
-static LaunchCfg launch_shape(const lidar_ctx* c, int64_t ray_tiles)
+// What the frames of a cast or sweep have in common
+struct FrameMix {
+    bool equal = false;      // every frame has the same number of tiles
+    bool subrays = false;    // some beam has several rays
+    int64_t ray_tiles = 0;   // 32-ray tiles in all, sub-rays counted
+};
+
+// Launch configuration of a cast or sweep.  As long as no caller has set
+// block_threads or blocks_per_sm, the library chooses how many threads stay
+// resident: few tiles end with their longest walks, which want the fewest
+// neighbours (512 threads a SM); many are bound by issue and want the most
+// warps (1,024 at 64 registers).  Measured on 152 SMs with the 4-wide walk, us,
+// 512 / 768 / 1,024 threads a SM, by ray tiles:
+//   8,192   128 x 2048 beams in 1M triangles 110 / 113 / 123, in a city 91 / 90 / 98
+//   14,400  16 frames of 16 channels in 1M triangles 166 / 150 / 153
+//   16,384  two frames of 128 channels 157 / 155 / 164, in a city 142 / 130 / 132
+//   24,576  three 221 / 206 / 214
+//   30,472  a rig of four sensors, two frames 283 / 257 / 256
+//   32,768  four frames 295 / 253 / 255, eight of 64 channels 278 / 239 / 233
+//   65,536  eight frames 580 / 489 / 456, in a city 516 / 440 / 416
+// A warp that claims 32 beams walks all their sub-rays, in several steps: there
+// are fewer pieces to balance, and more ray tiles count as few:
+//   14,336  seven sub-rays, 32 channels in a city 207 / 212 / 226, a sweep 236 / 242 / 244
+//   24,576  three, 128 channels 235 / 223 / 244
+//   28,672  seven, two frames of 32 channels 274 / 270 / 291
+//   57,344  seven, 128 channels 427 / 392 / 422, four sweeps of 64 490 / 441 / 427
+//   114,688 seven, two frames of 128 channels 779 / 691 / 672
+// 256-thread blocks took 1-8 % less than 128-thread ones at each.
+static LaunchCfg launch_shape(const lidar_ctx* c, const FrameMix& mix)
 {
     LaunchCfg cfg = c->cfg;
     if (!c->own_shape || cfg.traversal != 2) return cfg;
     const int64_t warps = (int64_t)c->num_sms * 16;  // resident at 512 threads a SM
+    const int64_t few = (mix.subrays ? 8 : 5) * warps, some = (mix.subrays ? 24 : 12) * warps;
     cfg.block_threads = 256;
-    cfg.blocks_per_sm = ray_tiles < 8 * warps ? 2 : (ray_tiles < 32 * warps ? 3 : 4);
+    cfg.blocks_per_sm = mix.ray_tiles < few ? 2 : (mix.ray_tiles < some ? 3 : 4);
     return cfg;
 }
-
-// What the frames of a cast have in common
-struct FrameMix {
-    bool equal = false;      // every frame has the same number of tiles
-    int64_t ray_tiles = 0;   // 32-ray tiles in all, sub-rays counted
-};
 
 // shared front half of the cast entry points
 // Frame records and tile prefix of a cast.  With `inl` and at most
@@ -761,6 +773,7 @@ static lidar_status prepare_frames(lidar_ctx* c, const lidar_frame* frames, int3
         off += c->slots[s].n_beams;
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
         mix->ray_tiles += (c->slots[s].n_beams + 31) / 32 * c->slots[s].dev.n_sub;
+        mix->subrays = mix->subrays || c->slots[s].dev.n_sub > 1;
     }
     mix->equal = true;
     for (int32_t k = 1; k < n_frames; ++k)
@@ -961,8 +974,8 @@ static lidar_status cast_impl(lidar_ctx* c, const lidar_scene* scene, const Fram
     R.overlap_refused = &refused;
     const cudaError_t le = launch_cast(c->stream, S, c->sensors_dev, frames_dev, n_frames, prefix_dev, n_tiles,
                                        c->table, seed, out, c->status_dev, c->work_counter,
-                                       launch_shape(c, mix.ray_tiles), c->num_sms, n_total, nullptr, comp, n_points_dev, points, &scattered, inl,
-                                       use_region ? &R : nullptr, mix.equal);
+                                       launch_shape(c, mix), c->num_sms, n_total, nullptr, comp, n_points_dev, points,
+                                       &scattered, inl, use_region ? &R : nullptr, mix.equal);
     if (refused != cudaSuccess)
         log_info(std::string("cast: overlapped launch refused (") + cudaGetErrorString(refused) +
                  "), launched after the previous cast instead");
@@ -1211,12 +1224,13 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
         off += c->slots[s].n_beams;
         tiles += (c->slots[s].n_beams + tr - 1) / tr;
     }
-    bool equal = true;
-    int64_t ray_tiles = 0;
+    FrameMix mix;
+    mix.equal = true;
     for (int32_t k = 0; k < n_frames; ++k) {
-        if (prefix[(size_t)k] * n_frames != tiles * k) equal = false;
+        if (prefix[(size_t)k] * n_frames != tiles * k) mix.equal = false;
         const SensorSlot& sl = c->slots[frames[k].sensor];
-        ray_tiles += (sl.n_beams + 31) / 32 * sl.dev.n_sub;
+        mix.ray_tiles += (sl.n_beams + 31) / 32 * sl.dev.n_sub;
+        mix.subrays = mix.subrays || sl.dev.n_sub > 1;
     }
     DeviceGuard g(c->device);
     // sweep records, then the tile prefix at a 256-byte boundary, in one block
@@ -1242,7 +1256,7 @@ lidar_status lidar_cast_sweep(lidar_ctx* c, const lidar_scene* scene, const lida
     // persistent tiles that follow the slots' ray orders and schedules
     LIDAR_CUDA(launch_sweep_tiles(c->stream, scene_dev(scene), c->sensors_dev, c->sweeps_dev, n_frames, prefix_dev,
                                   tiles, c->table, seed, to_beams_out(beams), echo, c->status_dev, c->work_counter,
-                                  launch_shape(c, ray_tiles), c->num_sms, equal));
+                                  launch_shape(c, mix), c->num_sms, mix.equal));
     return LIDAR_OK;
 }
 

@@ -166,3 +166,24 @@ def test_whose_shape_a_cast_runs(make):
         batch.free()
     finally:
         lid.close()
+
+
+@pytest.mark.parametrize("n_frames,n_subrays,blocks", [(10, 1, (2, 3)), (24, 1, (3, 4)), (8, 2, (2, 3)), (24, 2, (3, 4))])
+def test_where_the_chosen_shape_changes(make, n_frames, n_subrays, blocks):
+    """1,216 tiles of 32 beams a frame and one fewer, at the bounds for 152 SMs: 12,160 and 29,184 tiles of 32 rays,
+    with sub-rays 19,456 and 58,368."""
+    from paper_2208_10295_gb300 import Lidar
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the bounds depend on the number of SMs")
+    for off, want in zip((32, 0), blocks):
+        lid = Lidar(0, torch.cuda.Stream())
+        try:
+            w = _workload(n_frames, 1216, off, n_subrays)
+            scene = setup(lid, w)[0]
+            frames = w.frames[:n_frames]
+            beams = lid.alloc_beams(lid.total_beams(frames), ("valid",))
+            batch = lid.batch(frames)
+            assert _captured_shape(lid, batch, scene, w, beams) == (256, want)
+            batch.free()
+        finally:
+            lid.close()
