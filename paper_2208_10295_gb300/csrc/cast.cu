@@ -657,8 +657,7 @@ cudaError_t launch_cast(cudaStream_t s, const SceneDev& scene, const SensorDev* 
     const size_t stack_bytes = (size_t)kSharedStack * cfg.block_threads * sizeof(int2);
     const int bt = cfg.block_threads;
     cudaError_t e;
-    // (the bounds-checked build walks with 64-bit addresses throughout)
-    const bool far4 = kBoundsChecks || scene.n_nodes4 > kNearNodes4;
+    const bool far4 = scene.n_nodes4 > kNearNodes4;
     const int trav = cfg.traversal == 2 && far4 ? kTravFar4 : cfg.traversal;
     auto by_residency = [&](auto w, size_t smem) {
         constexpr int W = decltype(w)::value;

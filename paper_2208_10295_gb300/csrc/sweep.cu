@@ -255,8 +255,7 @@ cudaError_t launch_sweep_tiles(cudaStream_t s, const SceneDev& S, const SensorDe
     const int resident = cfg.block_threads * cfg.blocks_per_sm;
     const int bt = cfg.block_threads;
     const dim3 gd((unsigned)grid);
-    // node arrays too large for 32-bit offsets (and the bounds-checked build)
-    const bool far4 = kBoundsChecks || S.n_nodes4 > kNearNodes4;
+    const bool far4 = S.n_nodes4 > kNearNodes4;  // node arrays too large for 32-bit offsets
 #define LIDAR_SWEEP_LAUNCH(MB, EC)                                                                              \
     (far4 ? k_sweep_tiles<MB, EC, true> : k_sweep_tiles<MB, EC, false>)<<<gd, bt, 0, s>>>(                      \
         S, sensors_dev, frames_dev, n_frames, tile_prefix_dev, n_tiles, cfg.tile_rays, T, seed, out, echo,      \

@@ -443,8 +443,9 @@ __device__ __forceinline__ void sort2u(unsigned& a, unsigned& b)
 // instead of two and half the registers; kFar adds 64-bit addresses.  With the
 // fused slab distances above: 16 frames of 128 x 2048 beams in 1M triangles
 // 851 -> 836 us (fused) -> 820 us (offsets), four frames of seven sub-rays in a
-// 2.6M-triangle city 1447 -> 1413 -> 1356 us.
-constexpr int64_t kNearNodes4 = (int64_t)1 << 25;
+// 2.6M-triangle city 1447 -> 1413 -> 1356 us.  The bounds-checked build sets
+// the limit where small scenes lie on either side, so that it checks both.
+constexpr int64_t kNearNodes4 = kBoundsChecks ? (int64_t)1 << 14 : (int64_t)1 << 25;
 
 template <bool kFar, bool kCount = false>
 __device__ __forceinline__ bool trace_closest4(const SceneDev& S, const RayPre& p, float t_max, HitRec& h,
