@@ -128,8 +128,8 @@ lidar_status lidar_get_scene_info(const lidar_scene* scene, lidar_scene_info* ou
  *   method 1: PLOC, parallel locally-ordered clustering (Meister and Bittner,
  *             IEEE TVCG 2018) over the same Morton-ordered triangles: each
  *             cluster's nearest neighbour by union-box surface area within
- *             ploc_radius positions, mutual pairs merged, repeated; one host
- *             synchronisation per round.
+ *             ploc_radius positions, mutual pairs merged, repeated, all on the
+ *             device.
  * Applies to scenes built afterwards. */
 typedef struct {
     int32_t method;        /* 0 LBVH, 1 PLOC (default: about a third fewer node fetches per ray) */

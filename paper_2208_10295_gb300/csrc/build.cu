@@ -1545,7 +1545,6 @@ namespace {
 constexpr int kTreeletLeaves = 7;
 
 struct TreeletArgs {
-    const float4* tris;
     int n_leaves;
     int n_binary;
     float4* nodes;            // binary nodes, rewritten in place
@@ -2085,7 +2084,7 @@ size_t treelet_scratch_bytes(int64_t n_tris)
     return 5 * align256(n_tris * sizeof(int)) + 3 * align256(n_tris);
 }
 
-cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, float4* nodes, int* max_height_dev,
+cudaError_t restructure_treelets(cudaStream_t s, int64_t n, float4* nodes, int* max_height_dev,
                                  int rounds, float tri_cost, void* scratch, size_t scratch_bytes,
                                  unsigned long long* treelets_dev, int* status, AreaW area_w)
 {
@@ -2104,7 +2103,7 @@ cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, 
     uint8_t* mark = (uint8_t*)p; p += align256(n);
     uint8_t* up = (uint8_t*)p; p += align256(n);
     const int nb_blocks = (n_binary + 255) / 256;
-    TreeletArgs a{tris, (int)n, n_binary, nodes, parent_node, on_path, expect, visits, cost, mark, up, 0, treelets_dev,
+    TreeletArgs a{(int)n, n_binary, nodes, parent_node, on_path, expect, visits, cost, mark, up, 0, treelets_dev,
                   status, 1.0f, tri_cost, area_w};
     e = cudaMemsetAsync(on_path, 0, (size_t)(p - (char*)on_path), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(expect, 0, (size_t)((char*)cost - (char*)expect), s);

@@ -187,7 +187,7 @@ size_t collapse_scratch_bytes(int64_t n_binary, int sah_dp);
 // recomputes the root height; *treelets_dev receives the number of treelets
 // rewritten; a broken input tree records ST_BOUNDS in *status
 size_t treelet_scratch_bytes(int64_t n_tris);
-cudaError_t restructure_treelets(cudaStream_t s, const float4* tris, int64_t n, float4* nodes, int* max_height_dev,
+cudaError_t restructure_treelets(cudaStream_t s, int64_t n, float4* nodes, int* max_height_dev,
                                  int rounds, float tri_cost, void* scratch, size_t scratch_bytes,
                                  unsigned long long* treelets_dev, int* status,
                                  AreaW area_w = AreaW{1.0f, 1.0f, 1.0f});

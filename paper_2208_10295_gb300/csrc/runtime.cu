@@ -443,7 +443,7 @@ lidar_status lidar_scene_build(lidar_ctx* c, const float* verts, int64_t n_verts
                                    c->num_sms, c->coop, c->cfg.wait_ns, n_tris >= 2 ? c->build_method : 0,
                                    c->ploc_radius, c->area_w);
         if (e == cudaSuccess && c->treelet_rounds > 0)
-            e = restructure_treelets(c->stream, s->tris, n_tris, s->nodes, &c->build_dev->height, c->treelet_rounds,
+            e = restructure_treelets(c->stream, n_tris, s->nodes, &c->build_dev->height, c->treelet_rounds,
                                      c->tri_cost, c->scratch, c->scratch_bytes, &c->build_dev->treelets, c->status_dev,
                                      c->area_w);
         if (e == cudaSuccess)

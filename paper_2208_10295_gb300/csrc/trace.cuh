@@ -331,11 +331,10 @@ __device__ __forceinline__ bool trace_closest(const SceneDev& S, const RayPre& p
     return true;
 }
 
-// Slab test of the four child boxes of a 4-wide node (child boxes as SoA
-// float4 per plane), same rounding and NaN handling as child_boxes.
-// Packed FP32 pairs (sm_100+ f32x2 arithmetic): each lane of the pair is
-// rounded exactly like the scalar __fsub_rn / __fmul_rn, so the slab distances
-// are bit-identical to slab_t, with half the instructions.
+// Slab test of a wide node's child boxes (SoA, a float4 per plane of four), in
+// packed FP32 pairs (sm_100+ f32x2 arithmetic), two planes an instruction.  Its
+// distances are not those of child_boxes: SlabRay's constants keep every box
+// that holds a hit, and may keep one that child_boxes leaves out.
 __device__ __forceinline__ unsigned long long pack2(float a, float b)
 {
     unsigned long long r;
