@@ -64,26 +64,26 @@ POINT_BYTES = 12 + 4 + 4 + 12 + 2 + 4 + 4 + 4   # xyz, range, intensity, normal,
 # the cast kernel as the roofline times it (cfg1 frame, dense valid flags out,
 # L2 flushed before the launch), from one ncu capture, with the digest of the
 # kernel sources the capture ran.  Reported only while the sources still match.
-NCU_TRAFFIC = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
-               "bytes": 9_704_192 + 58_368, "l2_bytes": 3_410_835 * 32,
+NCU_TRAFFIC = {"sources": "ee01af58ca97c877", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
+               "bytes": 9_676_800 + 49_664, "l2_bytes": 3_411_089 * 32,
                "l1_global_load_bytes": 6_629_948 * 32}   # profiles/k_cast_cfg1_ncu_full.md
 # Binding-unit fractions of the same capture (ncu --set full of one launch):
 # L1/TEX throughput, issue-active and SM-active shares.
-NCU_UNITS = {"l1tex_throughput_pct": 45.6, "issue_active_pct": 42.3, "sm_active_pct": 71.1}
+NCU_UNITS = {"l1tex_throughput_pct": 45.5, "issue_active_pct": 42.6, "sm_active_pct": 71.8}
 # FP32 work of one launch of the cast kernel from ncu's SASS instruction
 # counters (sm__sass_thread_inst_executed_op_{ffma,fadd,fmul,ffma2,fadd2,fmul2,
 # fp32}_pred_on), FLOPs = 2 ffma + fadd + fmul + 4 ffma2 + 2 fadd2 + 2 fmul2 +
 # the remaining FP32 instructions (min/max, compares) once each.
-NCU_FP32 = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
+NCU_FP32 = {"sources": "ee01af58ca97c877", "tree": dict(treelet_rounds=2, area_weight=(1.0, 1.0, 0.23)),
             "fp32_flops": 499_329_365, "fp32_ops": 339_857_714,
             "counters": {"ffma": 22_224_867, "fadd": 12_038_981, "fmul": 34_606_334, "ffma2": 68_623_392,
                          "fadd2": 0, "fmul2": 0, "fp32_all": 271_234_322}}
 # profiles/k_cast_cfg1_fp32_counts.md
 # Binding-unit fractions of one city frame launch (ncu --set full,
 # profiles/k_cast_city_ncu_full.md), with the sources and tree it ran
-NCU_CITY_UNITS = {"sources": "d8742490fbd13b4a", "tree": dict(treelet_rounds=8, area_weight=(1.0, 1.0, 0.35)),
+NCU_CITY_UNITS = {"sources": "ee01af58ca97c877", "tree": dict(treelet_rounds=8, area_weight=(1.0, 1.0, 0.35)),
                   "kernel": "k_cast<0, 4, 2>",
-                  "issue_active_pct": 76.2, "l1tex_throughput_pct": 69.8, "fma_pipe_pct": 32.0, "alu_pipe_pct": 60.7}
+                  "issue_active_pct": 76.2, "l1tex_throughput_pct": 70.0, "fma_pipe_pct": 32.1, "alu_pipe_pct": 60.9}
 KERNEL_SOURCES = ("cast.cu", "shade.cuh", "trace.cuh", "common.cuh", "philox.cuh")
 # DRAM traffic (read + write) of one launch of the one-pass adjoint on the
 # 16-frame tape, from one ncu capture (profiles/k_adj_cfg3_ncu_full.md),

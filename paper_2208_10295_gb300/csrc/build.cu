@@ -1981,7 +1981,8 @@ __global__ void __launch_bounds__(kBuildThreads) k_treelet_paths(TreeletArgs a)
 // and with one acquire-release arrival a level 1.14, 0.83, 0.60, 0.42, 0.32,
 // 0.30, 0.25, 0.24 ms.  (Looking kTreeletReach levels above every change, and
 // not only while it still moves the costs, took the whole load from 5.21 to
-// 5.31 ms; it is what makes the rounds those of a full evaluation.)  A stride between a warp's nodes, fewer lanes or more
+// 5.31 ms, a round 1.14, 0.84, 0.61, 0.44, 0.34, 0.30, 0.25, 0.24 ms; it is what
+// makes the rounds those of a full evaluation.)  A stride between a warp's nodes, fewer lanes or more
 // nodes a warp all took longer: neighbours share the climb.
 __global__ void __launch_bounds__(kTreeletThreads, kTreeletBlocks) k_treelet_round(TreeletArgs a)
 {
